@@ -274,7 +274,8 @@ __device__ __forceinline__ bool try_tile(const RunDev &rd, int kt, char *smem, i
                                          const int *split)
 {
     if (rd.l != L || kt != KT) return false;
-    tile_2d<L, KT, float>(rd, smem, tile, rd.tt, split);  // the descriptor copy holds the tables
+    // the descriptor copy holds the tables
+    tile_2d<L, KT, float, false, SharedSplit>(rd, smem, tile, rd.tt, SharedSplit{split});
     return true;
 }
 

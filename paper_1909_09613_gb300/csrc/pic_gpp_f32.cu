@@ -20,7 +20,7 @@ cudaError_t go(const RunDev &rd, cudaStream_t st)
     auto k = rd.det ? k_gpp2d<L, KT, true> : k_gpp2d<L, KT, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)rd.ntiles, 256, smem, st>>>(rd);
+    k<<<dim3((unsigned)rd.ntiles, tile_parts(rd)), 256, smem, st>>>(rd);
     return cudaGetLastError();
 }
 

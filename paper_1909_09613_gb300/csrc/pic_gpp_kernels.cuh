@@ -949,14 +949,27 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     }
 }
 
-// All particles of one tile (both species), 2D.  tt_shared as in stage2d_carve.  split (in
-// shared memory: part, parts), when given with parts > 1: only that part of every species'
-// particles of the tile (a contiguous share of its range) -- the batched kernel splits the
-// heavy tiles of a small run set over several CTAs, each staging the tile and adding its own
-// share of the current.  (Read where used, so that it holds no registers across the tile.)
-template <int L, int KT, typename R, bool DET = false>
+// Which share of a tile's particles a CTA takes: part() of parts(), read where used so that it
+// holds no registers across the tile.  A single run's launch puts the part in blockIdx.y
+// (tile_parts chooses how many); the batched kernel keeps it in shared memory beside its work
+// item.
+struct GridSplit {
+    __device__ __forceinline__ int part() const { return (int)blockIdx.y; }
+    __device__ __forceinline__ int parts() const { return (int)gridDim.y; }
+};
+struct SharedSplit {
+    const int *s;  // (part, parts)
+    __device__ __forceinline__ int part() const { return s[0]; }
+    __device__ __forceinline__ int parts() const { return s[1]; }
+};
+
+// All particles of one tile (both species), 2D.  tt_shared as in stage2d_carve.  With
+// split.parts() > 1 only that part of every species' particles of the tile (a contiguous share
+// of its range): a grid of few tiles, or a batch of few particles, is spread over several CTAs
+// per tile, each staging the tile and adding its own share of the current.
+template <int L, int KT, typename R, bool DET = false, typename Split = GridSplit>
 __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
-                        const TTable *tt_shared = nullptr, const int *split = nullptr)
+                        const TTable *tt_shared = nullptr, const Split split = Split())
 {
     Stage2D<R> st = stage2d_carve<R>(smem, rd.reg_nodes, tt_shared, DET);
     const int tx = (int)(tile % rd.ntile[0]);
@@ -969,8 +982,9 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
         const SpeciesDev &sp = rd.sp[s];
         const HotSp<R> hs = make_hotsp<R>(sp);
         int64_t a = sp.tile_start[tile], b = sp.tile_start[tile + 1];
-        if (split != nullptr && split[1] > 1) {  // (fewer than 2^27 particles per tile)
-            const int len = (int)(b - a), part = split[0], parts = split[1];
+        if (split.parts() > 1) {
+            const int64_t len = b - a;
+            const int part = split.part(), parts = split.parts();
             b = a + (len * (part + 1)) / parts;
             a += (len * part) / parts;
         }
@@ -991,8 +1005,10 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
                 particle_2d<L, KT, R, DET>(h, hs, st, p, p < cb, x0, y0);
             }
         } else {
-            // warp-uniform trip count: a warp's lanes take 32 consecutive particles
-            const int64_t wbase = a + (threadIdx.x & ~31);
+            // warp-uniform trip count: a warp's lanes take 32 consecutive particles.  The
+            // species start at different warps, so that a part of few particles does not queue
+            // its species one behind the other on the first warps.
+            const int64_t wbase = a + ((threadIdx.x + s * (blockDim.x / 2)) & (blockDim.x - 1) & ~31);
             for (int64_t q = wbase; q < b; q += blockDim.x) {
                 const int64_t p = q + (threadIdx.x & 31);
                 if (p + blockDim.x < b) {

@@ -7,6 +7,35 @@ namespace pic {
 bool build_ttable(int l, int scheme, double dtt, TTable *t);
 int ttable_eval_host(const TTable *t, int l, double delta, double *w);
 
+// CTAs per tile of a single run's 2D particle pass (tile_2d's split), from the tile and particle
+// counts.  A grid of few tiles left most SMs idle: 64x32 cells are 4 to 8 tiles, 256x128 are 64,
+// on 304 CTA slots (two per SM).  Every tile takes as many parts as fill the slots once, down to
+// one warp of each species per part (particle kernel, us, one CTA per tile -> this rule: FP64
+// 64x32 quadratic at 4 per cell 105 -> 21, FP32 50 -> 23, FP32 250x126 cubic at 8 per cell 85 ->
+// 44, FP32 256x128 quartic at 64 per cell 445 -> 173).  The FP64 form, bound by a pipe every CTA
+// of the SM shares, also splits a grid of few waves so that its last wave is short, while a part
+// keeps 256 particles of a species (512x256 cubic at 64 per cell: 7388 -> 6362 us); the FP32 form
+// loses there to the parts' extra stages and flushes (256 tiles: 421 us with one part, 432 with
+// two) and stays at one wave.
+inline unsigned tile_parts(const RunDev &rd)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess
+        || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    int64_t n = 0;
+    for (int s = 0; s < rd.nsp; ++s) n = rd.sp[s].n > n ? rd.sp[s].n : n;
+    const int64_t slots = 2 * (int64_t)sms, per_tile = (n + rd.ntiles - 1) / rd.ntiles;
+    int64_t parts = slots / rd.ntiles;
+    if (rd.prec == 0) {
+        const int64_t want = (8 * slots + rd.ntiles - 1) / rd.ntiles, most = per_tile / 256;
+        const int64_t p = want < most ? want : most;
+        if (p > parts) parts = p;
+    }
+    const int64_t most = (per_tile + 31) / 32;
+    if (parts > most) parts = most;
+    return (unsigned)(parts > 1 ? parts : 1);
+}
 // fused gather-push-deposit over all tiles of one run
 cudaError_t launch_gpp(const RunDev &rd, int kt, cudaStream_t st);
 size_t gpp_smem_bytes(const RunDev &rd);
