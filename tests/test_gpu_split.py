@@ -19,13 +19,16 @@ def _built():
 
 
 # (grid, spline order, particles of each species): fewer particles than a warp, one more than a
-# warp, an empty species, uneven species, and enough tiles that FP64 parts span several waves
-CASES = [((9, 7), 2, (1, 31)), ((64, 8), 3, (33, 0)), ((33, 17), 4, (257, 64)),
-         ((70, 9), 1, (5000, 130)), ((512, 128), 3, (300001, 299999))]
+# warp, an empty species and uneven species in both forms; and, FP64 form only (the FP32 form
+# never splits a grid of several waves, and its FP32 sums over the 150,000 particles of one cell
+# round by sqrt(150000) 2^-24 = 2e-5 of their size), parts that span several waves
+SMALL = [((9, 7), 2, (1, 31)), ((64, 8), 3, (33, 0)), ((33, 17), 4, (257, 64)),
+         ((70, 9), 1, (5000, 130))]
+CASES = ([c + (pic.PIC_FP64, 1e-12) for c in SMALL + [((512, 128), 3, (300001, 299999))]]
+         + [c + (pic.PIC_FP32_MIXED, 2e-6) for c in SMALL])
 
 
-@pytest.mark.parametrize("grid,l,counts", CASES)
-@pytest.mark.parametrize("prec,tol", [(pic.PIC_FP64, 1e-12), (pic.PIC_FP32_MIXED, 2e-6)])
+@pytest.mark.parametrize("grid,l,counts,prec,tol", CASES)
 def test_split_tiles_match_oracle(grid, l, counts, prec, tol):
     rng = np.random.default_rng(sum(counts))
     n = (grid[0], grid[1], 1)
