@@ -26,10 +26,24 @@ struct TTable {
     int Rint;         // floor(R)
     double Rfrac;     // R - floor(R)
     double phib;      // interior breakpoint (0 if none)
-    double coef[2][PIC_TK_MAX][5];
+    union {
+        double coef[2][PIC_TK_MAX][5];
+        // 2D FP64 form: the coefficients of the polynomial in s = t / h, h the length of the
+        // sub-interval, in units of 2^-59 (pic_fixed.cuh)
+        int64_t ci[2][PIC_TK_MAX][5];
+    };
     float Rfrac_f, phib_f;
-    // coef in FP32, grouped for vector loads: cf4[p][m][g] = coefficient m of nodes 4g .. 4g + 3
-    float4 cf4[2][5][2];
+    union {
+        // FP32 form: coef in FP32, grouped for vector loads: cf4[p][m][g] = coefficient m of
+        // nodes 4g .. 4g + 3
+        float4 cf4[2][5][2];
+        // 2D FP64 form: Rfrac and phib in units of 2^-64, and 1 / h = 2^shift (1 + invm1) per
+        // sub-interval (invm1 in units of 2^-62)
+        struct {
+            uint64_t rfrac, phib, invm1[2];
+            int shift[2];
+        } fx;
+    };
 };
 
 // Scratch of the tile sort (one set per run; the species are sorted one after the other).
@@ -59,14 +73,6 @@ struct SpeciesDev {
     void *pos_alt[3];
     void *mom_alt[3];
     int32_t *cell_alt;
-    // FP64 2D: the B-spline weights of each particle at its stored position, l + 1 per axis at
-    // wc[(a (l + 1) + k) wc_stride + p], written by every step for the next one, whose
-    // old-position deposit weights they are (bit-identical by construction of the move).
-    // wc_mode: 0 no cache, 1 write only (the positions were loaded or re-ordered since the
-    // last step), 2 read and write.
-    double *wc;
-    int64_t wc_stride;
-    int wc_mode;
 };
 
 // Exact quotient n / d for 0 <= n < 2^31 and 1 <= d < 2^31 by one multiply and a shift:

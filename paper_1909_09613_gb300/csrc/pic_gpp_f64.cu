@@ -1,5 +1,5 @@
-// Instantiations of the fused particle pass, double arithmetic.
-#include "pic_gpp_kernels.cuh"
+// Instantiations of the 2D particle pass of the plain FP64 form.
+#include "pic_gpp_fx.cuh"
 #include "pic_launch.h"
 
 namespace pic {
@@ -10,13 +10,13 @@ template <int L, int KT, bool DET>
 __global__ void __launch_bounds__(256, 2) k_gpp2d(const __grid_constant__ RunDev rd)
 {
     extern __shared__ __align__(16) char smem[];
-    tile_2d<L, KT, double, DET>(rd, smem, blockIdx.x);
+    tile_fx<L, KT, DET>(rd, smem, blockIdx.x);
 }
 
 template <int L, int KT>
 cudaError_t go(const RunDev &rd, cudaStream_t st)
 {
-    const size_t smem = stage2d_bytes<double>(rd.reg_nodes, rd.l);
+    const size_t smem = stage_fx_bytes(rd.reg_nodes);
     auto k = rd.det ? k_gpp2d<L, KT, true> : k_gpp2d<L, KT, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -41,7 +41,7 @@ cudaError_t launch_gpp_f64(const RunDev &rd, int kt, cudaStream_t st)
 
 size_t gpp_smem_bytes_f64(const RunDev &rd)
 {
-    return rd.dim == 2 ? stage2d_bytes<double>(rd.reg_nodes, rd.l) : 0;
+    return rd.dim == 2 ? stage_fx_bytes(rd.reg_nodes) : 0;
 }
 
 }  // namespace pic

@@ -154,17 +154,10 @@ __device__ void stage2d_load(const RunDev &rd, const Stage2D<R> &st, int x0, int
         const int gy = wrap_idx(y0 - rd.pre[1] + ry, rd.n[1]);
         const int64_t g = (int64_t)gy * rd.n[0] + gx;
         typename Vec2<R>::T a, b;
-        if constexpr (sizeof(R) == 4) {
-            a.x = __ldg(rd.Fs[0] + g); a.y = __ldg(rd.Fs[4] + g);
-            b.x = __ldg(rd.Fs[1] + g); b.y = __ldg(rd.Fs[3] + g);
-            st.e3[n] = __ldg(rd.Fs[2] + g);
-            st.b3[n] = __ldg(rd.Fs[5] + g);
-        } else {
-            a.x = __ldg(rd.F[0] + g); a.y = __ldg(rd.F[4] + g);
-            b.x = __ldg(rd.F[1] + g); b.y = __ldg(rd.F[3] + g);
-            st.e3[n] = __ldg(rd.F[2] + g);
-            st.b3[n] = __ldg(rd.F[5] + g);
-        }
+        a.x = __ldg(rd.Fs[0] + g); a.y = __ldg(rd.Fs[4] + g);
+        b.x = __ldg(rd.Fs[1] + g); b.y = __ldg(rd.Fs[3] + g);
+        st.e3[n] = __ldg(rd.Fs[2] + g);
+        st.b3[n] = __ldg(rd.Fs[5] + g);
         st.pa[n] = a;
         st.pb[n] = b;
         if (st.q1) {
@@ -251,7 +244,8 @@ __device__ __forceinline__ void atomic_add_pair(float *p, float a, float b)
 
 // One lane's Esirkepov window (Sec. 1: W_x = DSx (S0y + DSy/2) summed along x, W_y likewise,
 // W_z = S0x S0y + DSx S0y/2 + S0x DSy/2 + DSx DSy/3) added to the shared current tile with
-// atomics (WY as in deposit_lane_global below); DET: as fixed-point words (RunDev::det).
+// atomics; WY = false when no
+// lane of the warp changed its y window base, so that row l + 1 carries exact zeros; DET: as fixed-point words (RunDev::det).
 template <int L, typename R, bool WY = true, bool DET = false>
 __device__ __forceinline__ void deposit_lane(const Stage2D<R> &st, int RX, int jx0, int jy0, R kx,
                                              R ky, R kz, const R *px, const R *py, const R *Ax,
@@ -279,57 +273,6 @@ __device__ __forceinline__ void deposit_lane(const Stage2D<R> &st, int RX, int j
     }
 }
 
-// One lane's Esirkepov window added straight to the global FP64 current (FP64 form).  The
-// reductions (red.global.add.f64) are performed by L2, so unlike shared-memory FP64 atomics
-// (compare-and-swap loops around a DADD) they take no issue slots of the SM's FP64 pipe, which
-// bounds this form.  gx0, gy0: global node of the window's first column and row (unwrapped).
-// WY = false when no lane of the warp changed its y window base: row l + 1 then carries exact
-// zeros (S0y = DSy = 0) and is skipped.
-template <int L, typename R, typename Hot, bool WY = true, bool DET = false>
-__device__ __forceinline__ void deposit_lane_global(const Hot &h, int gx0, int gy0, R kx, R ky,
-                                                    R kz, const R *px, const R *py, const R *Ax,
-                                                    const R *Ay, const R *Bx,
-                                                    const AxisS<L, R> &Sy)
-{
-    int gx[L + 2];
-    int64_t gy[L + 2];
-#pragma unroll
-    for (int k = 0; k < L + 2; ++k) {
-        gx[k] = wrap_near(gx0 + k, h.n0);
-        gy[k] = (int64_t)wrap_near(gy0 + k, h.n1) * h.n0;
-    }
-#pragma unroll
-    for (int b = 0; b < (WY ? L + 2 : L + 1); ++b) {
-        const R ayk = kx * Ay[b];
-        const R pyk = (b <= L) ? ky * py[b] : R(0);
-        const R zs = kz * Sy.s0[b], zd = kz * Sy.ds[b];
-#pragma unroll
-        for (int a = 0; a < L + 2; ++a) {
-            const int64_t g = gy[b] + gx[a];
-            if constexpr (DET) {
-                unsigned long long hi, lo;
-                if (a <= L) {
-                    det_words64((double)(ayk * px[a]), h.dinv64, hi, lo);
-                    atomicAdd((unsigned long long *)(h.J0 + g), hi);
-                    atomicAdd(h.Jlo0 + g, lo);
-                }
-                if (b <= L) {
-                    det_words64((double)(pyk * Ax[a]), h.dinv64, hi, lo);
-                    atomicAdd((unsigned long long *)(h.J1 + g), hi);
-                    atomicAdd(h.Jlo1 + g, lo);
-                }
-                det_words64((double)(zs * Ax[a] + zd * Bx[a]), h.dinv64, hi, lo);
-                atomicAdd((unsigned long long *)(h.J2 + g), hi);
-                atomicAdd(h.Jlo2 + g, lo);
-            } else {
-                if (a <= L) atomicAdd(h.J0 + g, (double)(ayk * px[a]));
-                if (b <= L) atomicAdd(h.J1 + g, (double)(pyk * Ax[a]));
-                atomicAdd(h.J2 + g, (double)(zs * Ax[a] + zd * Bx[a]));
-            }
-        }
-    }
-}
-
 // Scalars the particle loop uses, held in registers for the whole tile (a run descriptor in
 // shared or global memory would be re-read for every particle).
 struct Hot2D {
@@ -350,9 +293,6 @@ struct HotSp {
     void *pos0, *pos1, *mom0, *mom1, *mom2;
     int32_t *cell;
     double qmdt_half, kx0, kx1, kz;
-    double *wc;  // FP64 weight cache (SpeciesDev::wc)
-    int64_t wc_stride;
-    int wc_mode;
 };
 
 __device__ __forceinline__ Hot2D make_hot2d(const RunDev &rd)
@@ -385,7 +325,6 @@ __device__ __forceinline__ HotSp<R> make_hotsp(const SpeciesDev &sp)
     h.cell = sp.cell;
     h.qmdt_half = sp.qmdt_half;
     h.kx0 = sp.kx[0]; h.kx1 = sp.kx[1]; h.kz = sp.kz;
-    h.wc = sp.wc; h.wc_stride = sp.wc_stride; h.wc_mode = sp.wc_mode;
     return h;
 }
 
@@ -399,17 +338,6 @@ __device__ __forceinline__ void prefetch_particle(const HotSp<R> &hs, int64_t p)
     for (int i = 0; i < 6; ++i) {
         if (i == 5 && sizeof(R) == 8) break;  // the FP64 form has no cell array
         const char *a = (const char *)ptrs[i] + p * (i == 5 ? 4 : (int64_t)sizeof(R));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
-    }
-}
-
-// The cached old-position weights of a later iteration (FP64 form, 2 (l + 1) arrays).
-template <int L>
-__device__ __forceinline__ void prefetch_weights(const HotSp<double> &hs, int64_t p)
-{
-#pragma unroll
-    for (int i = 0; i < 2 * (L + 1); ++i) {
-        const double *a = hs.wc + (int64_t)i * hs.wc_stride + p;
         asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
     }
 }
@@ -715,22 +643,11 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     PState<R> s;
     int lx = 0, ly = 0;
     if (act) {
-        if constexpr (sizeof(R) == 4) {
-            const int c = __ldg(hs.cell + p);
-            s.c[1] = fast_div(c, h.dm, h.ds);
-            s.c[0] = c - s.c[1] * h.n0;
-            s.d[0] = __ldg((const float *)hs.pos0 + p);
-            s.d[1] = __ldg((const float *)hs.pos1 + p);
-        } else {
-            const double x0v = __ldg((const double *)hs.pos0 + p);
-            const double x1v = __ldg((const double *)hs.pos1 + p);
-            const double f0 = floor(x0v), f1 = floor(x1v);
-            // in [0, n) by construction; the clamp keeps a non-finite position's index valid
-            s.c[0] = min(max((int)f0, 0), h.n0 - 1);
-            s.c[1] = min(max((int)f1, 0), h.n1 - 1);
-            s.d[0] = x0v - f0;
-            s.d[1] = x1v - f1;
-        }
+        const int c = __ldg(hs.cell + p);
+        s.c[1] = fast_div(c, h.dm, h.ds);
+        s.c[0] = c - s.c[1] * h.n0;
+        s.d[0] = __ldg((const float *)hs.pos0 + p);
+        s.d[1] = __ldg((const float *)hs.pos1 + p);
         s.c[2] = 0;
         s.u[0] = __ldg((const R *)hs.mom0 + p);
         s.u[1] = __ldg((const R *)hs.mom1 + p);
@@ -758,62 +675,7 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
 
     // ---- gather (Eq. interpolation-EB-real-mod; MC when the tables hold W_l) ----
     R E[3], B[3];
-    if constexpr (sizeof(R) == 4) {
-        gather_2d_x2<L, KT>(st, wx, wy, sx, sy, RX, E, B);
-    } else {
-        // (E1, B2): W along x (half nodes), T along y (integer nodes)
-        R e1 = R(0), b2 = R(0);
-#pragma unroll
-        for (int b = 0; b < KT; ++b) {
-            const int row = (sy + wy.bt + b) * RX + sx + wx.bh;
-            R re = R(0), rb = R(0);
-#pragma unroll
-            for (int a = 0; a <= L; ++a) {
-                const typename Vec2<R>::T v = st.pa[row + a];
-                re += wx.wh[a] * v.x;
-                rb += wx.wh[a] * v.y;
-            }
-            e1 += wy.wt[b] * re;
-            b2 += wy.wt[b] * rb;
-        }
-        // (E2, B1): T along x, W along y
-        R e2 = R(0), b1 = R(0);
-#pragma unroll
-        for (int b = 0; b <= L; ++b) {
-            const int row = (sy + wy.bh + b) * RX + sx + wx.bt;
-            R re = R(0), rb = R(0);
-#pragma unroll
-            for (int a = 0; a < KT; ++a) {
-                const typename Vec2<R>::T v = st.pb[row + a];
-                re += wx.wt[a] * v.x;
-                rb += wx.wt[a] * v.y;
-            }
-            e2 += wy.wh[b] * re;
-            b1 += wy.wh[b] * rb;
-        }
-        // E3: T T
-        R e3 = R(0);
-#pragma unroll
-        for (int b = 0; b < KT; ++b) {
-            const int row = (sy + wy.bt + b) * RX + sx + wx.bt;
-            R r = R(0);
-#pragma unroll
-            for (int a = 0; a < KT; ++a) r += wx.wt[a] * st.e3[row + a];
-            e3 += wy.wt[b] * r;
-        }
-        // B3: W W
-        R b3 = R(0);
-#pragma unroll
-        for (int b = 0; b <= L; ++b) {
-            const int row = (sy + wy.bh + b) * RX + sx + wx.bh;
-            R r = R(0);
-#pragma unroll
-            for (int a = 0; a <= L; ++a) r += wx.wh[a] * st.b3[row + a];
-            b3 += wy.wh[b] * r;
-        }
-        E[0] = e1; E[1] = e2; E[2] = e3;
-        B[0] = b1; B[1] = b2; B[2] = b3;
-    }
+    gather_2d_x2<L, KT>(st, wx, wy, sx, sy, RX, E, B);
 
     // ---- Boris push ----
     const R ig = boris<R>(R(hs.qmdt_half), E, B, s.u);
@@ -829,26 +691,13 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
 
     // ---- Esirkepov deposit ----
     AxisS<L, R> Sx, Sy;
-    if constexpr (sizeof(R) == 4) {
-        axis_shapes_dd<L, true>(s.d[0], dl[0], Sx);  // all 32 lanes take part
-        axis_shapes_dd<L, true>(s.d[1], dl[1], Sy);
-    } else {
-        // old-position weights: from the cache the previous step wrote at this particle's
-        // stored position (bit-identical to evaluating them), else evaluated.  (l = 4 keeps
-        // evaluating: its cache would not fit the register budget of two CTAs per SM.)
-        double *wc = (L <= 3 && act && hs.wc_mode != 0) ? hs.wc + p : nullptr;
-        const double *wr = hs.wc_mode == 2 ? wc : nullptr;
-        const int64_t ws = hs.wc_stride;
-        axis_shapes<L, R>(s.d[0], shv[0], o[0], Sx, wr, wc, ws);
-        axis_shapes<L, R>(s.d[1], shv[1], o[1], Sy, wr ? wr + (L + 1) * ws : nullptr,
-                          wc ? wc + (L + 1) * ws : nullptr, ws);
-    }
-    // the FP32 warp-collective deposit carries idle lanes with zero weight; the FP64 form
-    // deposits active lanes only, and saves the three products
-    const R wgt = (sizeof(R) == 8 || act) ? R(1) : R(0);
-    const R kx = (sizeof(R) == 8) ? R(hs.kx0) : wgt * R(hs.kx0);
-    const R ky = (sizeof(R) == 8) ? R(hs.kx1) : wgt * R(hs.kx1);
-    const R kz = ((sizeof(R) == 8) ? R(hs.kz) : wgt * R(hs.kz)) * s.u[2] * ig;
+    axis_shapes_dd<L, true>(s.d[0], dl[0], Sx);  // all 32 lanes take part
+    axis_shapes_dd<L, true>(s.d[1], dl[1], Sy);
+    // the warp-collective deposit carries idle lanes with zero weight
+    const R wgt = act ? R(1) : R(0);
+    const R kx = wgt * R(hs.kx0);
+    const R ky = wgt * R(hs.kx1);
+    const R kz = wgt * R(hs.kz) * s.u[2] * ig;
     const R third = R(1) / R(3);
     // W_x = DSx (S0y + DSy/2), prefix along x; W_y = DSy (S0x + DSx/2), prefix along y;
     // W_z = S0x S0y + DSx S0y/2 + S0x DSy/2 + DSx DSy/3 = S0y Ax + DSy Bx.
@@ -866,7 +715,7 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     }
     const int jx0 = sx + Sx.wb, jy0 = sy + Sy.wb;
 
-    if constexpr (sizeof(R) == 4) {
+    {
         // Warp-collective path (cell-major order): lanes whose windows start at most SXM nodes
         // apart in x and SYM in y (up to three or four neighbouring cells along a row) form a
         // group; the group's current is a sum of per-lane outer products on a common block
@@ -914,24 +763,6 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
                                                            kz, px, py, Ax, Ay, Bx, Sy);
         }
         }
-    } else {
-        // a drift along x1 rarely moves the y window: skip its empty last row warp-uniformly
-        const bool wide = __any_sync(0xffffffffu, act && Sy.wide);
-        const int gx0 = x0 - h.pre0 + jx0, gy0 = y0 - h.pre1 + jy0;
-        if (!act) {
-        } else if (DET) {
-            if (wide)
-                deposit_lane_global<L, R, Hot2D, true, true>(h, gx0, gy0, kx, ky, kz, px, py, Ax,
-                                                             Ay, Bx, Sy);
-            else
-                deposit_lane_global<L, R, Hot2D, false, true>(h, gx0, gy0, kx, ky, kz, px, py,
-                                                              Ax, Ay, Bx, Sy);
-        } else if (wide) {
-            deposit_lane_global<L, R, Hot2D, true>(h, gx0, gy0, kx, ky, kz, px, py, Ax, Ay, Bx, Sy);
-        } else {
-            deposit_lane_global<L, R, Hot2D, false>(h, gx0, gy0, kx, ky, kz, px, py, Ax, Ay, Bx,
-                                                    Sy);
-        }
     }
     if (!act) return;
 
@@ -939,14 +770,9 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     ((R *)hs.mom0)[p] = s.u[0];
     ((R *)hs.mom1)[p] = s.u[1];
     ((R *)hs.mom2)[p] = s.u[2];
-    if constexpr (sizeof(R) == 4) {
-        hs.cell[p] = cn[1] * h.n0 + cn[0];
-        ((float *)hs.pos0)[p] = o[0];
-        ((float *)hs.pos1)[p] = o[1];
-    } else {
-        ((double *)hs.pos0)[p] = xs[0];  // = cn + o
-        ((double *)hs.pos1)[p] = xs[1];
-    }
+    hs.cell[p] = cn[1] * h.n0 + cn[0];
+    ((float *)hs.pos0)[p] = o[0];
+    ((float *)hs.pos1)[p] = o[1];
 }
 
 // Which share of a tile's particles a CTA takes: part() of parts(), read where used so that it
@@ -963,7 +789,18 @@ struct SharedSplit {
     __device__ __forceinline__ int parts() const { return s[1]; }
 };
 
-// All particles of one tile (both species), 2D.  tt_shared as in stage2d_carve.  With
+template <typename Split>
+__device__ __forceinline__ void split_range(const Split &split, int64_t &a, int64_t &b)
+{
+    if (split.parts() > 1) {
+        const int64_t len = b - a;
+        const int part = split.part(), parts = split.parts();
+        b = a + (len * (part + 1)) / parts;
+        a += (len * part) / parts;
+    }
+}
+
+// All particles of one tile (both species), 2D FP32 form.  tt_shared as in stage2d_carve.  With
 // split.parts() > 1 only that part of every species' particles of the tile (a contiguous share
 // of its range): a grid of few tiles, or a batch of few particles, is spread over several CTAs
 // per tile, each staging the tile and adding its own share of the current.
@@ -982,13 +819,8 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
         const SpeciesDev &sp = rd.sp[s];
         const HotSp<R> hs = make_hotsp<R>(sp);
         int64_t a = sp.tile_start[tile], b = sp.tile_start[tile + 1];
-        if (split.parts() > 1) {
-            const int64_t len = b - a;
-            const int part = split.part(), parts = split.parts();
-            b = a + (len * (part + 1)) / parts;
-            a += (len * part) / parts;
-        }
-        if constexpr (sizeof(R) == 4) {
+        split_range(split, a, b);
+        {
             // every warp takes a contiguous chunk of the tile's particles of this species (for a
             // uniform plasma in the cell-major order, one row of cells), so that the warps'
             // frames, a row apart, rarely race for the same nodes of the tile: 5.53 -> 5.38 ms
@@ -1004,26 +836,10 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
                 if (p + 32 < cb) prefetch_particle<R>(hs, p + 32);
                 particle_2d<L, KT, R, DET>(h, hs, st, p, p < cb, x0, y0);
             }
-        } else {
-            // warp-uniform trip count: a warp's lanes take 32 consecutive particles.  The
-            // species start at different warps, so that a part of few particles does not queue
-            // its species one behind the other on the first warps.
-            const int64_t wbase = a + ((threadIdx.x + s * (blockDim.x / 2)) & (blockDim.x - 1) & ~31);
-            for (int64_t q = wbase; q < b; q += blockDim.x) {
-                const int64_t p = q + (threadIdx.x & 31);
-                if (p + blockDim.x < b) {
-                    prefetch_particle<R>(hs, p + blockDim.x);
-                    if constexpr (sizeof(R) == 8 && L <= 3)
-                        if (hs.wc_mode == 2) prefetch_weights<L>(hs, p + blockDim.x);
-                }
-                particle_2d<L, KT, R, DET>(h, hs, st, p, p < b, x0, y0);
-            }
         }
-        if constexpr (sizeof(R) == 4) {  // the FP64 form deposits to global memory directly
-            __syncthreads();
-            stage2d_flush<R>(rd, st, x0, y0);
-            __syncthreads();
-        }
+        __syncthreads();
+        stage2d_flush<R>(rd, st, x0, y0);
+        __syncthreads();
     }
 }
 

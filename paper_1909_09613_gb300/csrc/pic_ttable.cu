@@ -100,6 +100,37 @@ static ld tfun_deriv(int l, ld dtt, ld y, ld y_loc, int m)
             - bspline_deriv(l - 1, y - dtt, y_loc - dtt, m - 1)) / (2 * dtt);
 }
 
+// Taylor coefficients c[p][k][m] of node k's weight about the left end of sub-interval p.
+static void taylor_coefs(int l, int scheme, ld dtt, ld R, ld phib, int K,
+                         ld (*c)[PIC_TK_MAX][5])
+{
+    for (int p = 0; p < 2; ++p) {
+        const ld a = p ? phib : 0;
+        const ld b = (p == 0 && phib > 0) ? phib : 1;
+        for (int k = 0; k < K; ++k) {
+            const ld y0 = R - 1 + a - k;
+            const ld ymid = R - 1 + (a + b) / 2 - k;
+            ld fact = 1;
+            for (int m = 0; m <= l; ++m) {
+                if (m > 0) fact *= m;
+                ld v;
+                if (scheme == 1) v = tfun_deriv(l, dtt, y0, ymid, m);
+                else v = bspline_deriv(l, y0, ymid, m);
+                c[p][k][m] = v / fact;
+            }
+        }
+    }
+}
+
+// Interior breakpoint frac(-2 dtt) of the WT weights (0: none).
+static ld breakpoint(int scheme, ld dtt)
+{
+    if (scheme != 1) return 0;
+    ld f = -2 * dtt;
+    f = f - std::floor((double)f);
+    return f > 1e-15 && f < 1 - 1e-15 ? f : 0;
+}
+
 // Build the table of one axis.  scheme 1 = WT (T_l), 0 = MC (W_l at integer nodes).
 bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
 {
@@ -118,29 +149,13 @@ bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
     t->K = K;
     t->Rint = (int)std::floor((double)R);
     t->Rfrac = (double)(R - t->Rint);
-    ld phib = 0;
-    if (scheme == 1) {
-        ld f = -2 * dtt;
-        f = f - std::floor((double)f);
-        if (f > 1e-15 && f < 1 - 1e-15) phib = f;
-    }
+    const ld phib = breakpoint(scheme, dtt);
     t->phib = (double)phib;
-    for (int p = 0; p < 2; ++p) {
-        const ld a = p ? phib : 0;
-        const ld b = (p == 0 && phib > 0) ? phib : 1;
-        for (int k = 0; k < K; ++k) {
-            const ld y0 = R - 1 + a - k;
-            const ld ymid = R - 1 + (a + b) / 2 - k;
-            ld fact = 1;
-            for (int m = 0; m <= l; ++m) {
-                if (m > 0) fact *= m;
-                ld v;
-                if (scheme == 1) v = tfun_deriv(l, dtt, y0, ymid, m);
-                else v = bspline_deriv(l, y0, ymid, m);
-                t->coef[p][k][m] = (double)(v / fact);
-            }
-        }
-    }
+    ld c[2][PIC_TK_MAX][5];
+    taylor_coefs(l, scheme, dtt, R, phib, K, c);
+    for (int p = 0; p < 2; ++p)
+        for (int k = 0; k < K; ++k)
+            for (int m = 0; m <= l; ++m) t->coef[p][k][m] = (double)c[p][k][m];
     for (int p = 0; p < 2; ++p)
         for (int m = 0; m < 5; ++m)
             for (int g = 0; g < 2; ++g) {
@@ -156,6 +171,33 @@ bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
     // the float split must reproduce the same breakpoint ordering
     if (t->Rfrac_f >= 1.0f) return false;
     return true;
+}
+
+// The fixed-point form of a table (2D FP64 form), in place of its FP64 coefficients; scheme and
+// dtt as build_ttable had them.
+void fix_ttable(int l, int scheme, double dtt, TTable *t)
+{
+    const ld R = scheme == 1 ? (ld)l / 2 + (ld)dtt : (ld)(l + 1) / 2;
+    const ld phib = breakpoint(scheme, dtt);
+    ld c[2][PIC_TK_MAX][5];
+    taylor_coefs(l, scheme, dtt, R, phib, t->K, c);
+    std::memset(&t->fx, 0, sizeof(t->cf4));
+    std::memset(t->ci, 0, sizeof(t->ci));
+    t->fx.rfrac = (uint64_t)std::ldexp(R - t->Rint, 64);
+    t->fx.phib = (uint64_t)std::ldexp(phib, 64);
+    for (int p = 0; p < 2; ++p) {
+        const ld h = p ? 1 - phib : (phib > 0 ? phib : 1);
+        // 2^shift <= 1 / h < 2^(shift + 1)
+        int sh = 0;
+        while (sh < 62 && std::ldexp(h, sh + 1) <= 1) ++sh;
+        t->fx.shift[p] = sh;
+        t->fx.invm1[p] = (uint64_t)std::ldexp(1 / std::ldexp(h, sh) - 1, 62);
+        for (int k = 0; k < t->K; ++k) {
+            ld hm = 1;
+            for (int m = 0; m <= l; ++m, hm *= h)
+                t->ci[p][k][m] = (int64_t)std::llround(std::ldexp(c[p][k][m] * hm, 59));
+        }
+    }
 }
 
 // Host evaluation of a table (same arithmetic as the device code, in double).
