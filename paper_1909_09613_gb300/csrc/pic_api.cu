@@ -453,9 +453,11 @@ int pic_create(const int32_t grid[3], const double dx[3], double dt, int spline_
     c->kt = 0;
     for (int a = 0; a < 3; ++a) {
         if (a >= dim) { build_ttable(spline_order, PIC_SCHEME_MC, 0.5, &rd.tt[a]); continue; }
-        if (!build_ttable(spline_order, scheme, rd.dtt[a], &rd.tt[a])) { delete c; return PIC_ECFL; }
+        if (!build_ttable(spline_order, scheme, rd.dtt[a], &rd.tt[a], dim == 2 && rd.prec == PIC_FP64)) {
+            delete c;
+            return PIC_ECFL;
+        }
         c->kt = std::max(c->kt, rd.tt[a].K);
-        if (dim == 2 && rd.prec == PIC_FP64) fix_ttable(spline_order, scheme, rd.dtt[a], &rd.tt[a]);
     }
     // sort interval and staged region
     double dmax = 0.0;

@@ -82,6 +82,16 @@ PIC_HD int decode_position(uint64_t bits, uint64_t &frac)
     return s <= 52 ? (int)(m >> s) : 0;
 }
 
+// An FP32 in-cell offset in [0, 1) in units of 2^-64, exact down to offsets of 2^-40.  A
+// non-finite offset gives some value.
+PIC_HD uint64_t offset_fixed(uint32_t bits)
+{
+    const int e = (int)(bits >> 23) & 0xff;
+    const uint64_t m = (bits & 0x7fffffu) | 0x800000u;
+    const int s = e - 86;
+    return s >= 0 ? m << (s < 40 ? s : 40) : (s > -24 && e > 0 ? m >> -s : 0);
+}
+
 // W_l at the l + 1 nodes (bspline<L> in U62), p = psi in U62, below 1.
 template <int L>
 PIC_HD void bspline62(uint64_t p, uint64_t *w)
@@ -192,6 +202,19 @@ PIC_HD uint64_t to_fp64_bits(uint64_t v, uint32_t top)
     const uint64_t m = (((uint64_t)hi << 32 | lo) >> 11) + ((lo >> 10) & 1);
     return m + ((uint64_t)(top - ((uint32_t)lz << 20)) << 32);
 }
+
+#ifdef __CUDACC__
+// *p += v (a U62, its scale's sign and exponent in top) as an FP64 reduction performed by L2;
+// nothing for v = 0.  Predicated, not branched around: the compiler's branch per contribution
+// cost more instructions than the conversion it skips.
+__device__ __forceinline__ void red_fixed(double *p, uint64_t v, uint32_t top)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u64 p, %2, 0;\n\t"
+                 "@p red.global.add.f64 [%0], %1;\n\t}"
+                 ::"l"(p), "d"(__longlong_as_double((int64_t)to_fp64_bits(v, top))), "l"(v)
+                 : "memory");
+}
+#endif
 
 // A field value as biased fixed point for a tile whose largest magnitude has the exponent field
 // emax: round(F 2^(59 - E)) + 2^59 with |F| < 2^E, E = emax - 1022.

@@ -175,19 +175,14 @@ template <bool DET>
 __device__ __forceinline__ void add_current_fx(double *J, unsigned long long *Jlo, int g,
                                                uint64_t v, uint32_t top, double dinv)
 {
-    const double c = __longlong_as_double((int64_t)to_fp64_bits(v, top));
     if constexpr (DET) {
         if (v == 0) return;
         unsigned long long hi, lo;
-        det_words64(c, dinv, hi, lo);
+        det_words64(__longlong_as_double((int64_t)to_fp64_bits(v, top)), dinv, hi, lo);
         atomicAdd((unsigned long long *)(J + g), hi);
         atomicAdd(Jlo + g, lo);
     } else {
-        // predicated, not branched around (the compiler's branch per contribution cost more
-        // instructions than the conversion it skips)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u64 p, %2, 0;\n\t"
-                     "@p red.global.add.f64 [%0], %1;\n\t}"
-                     ::"l"(J + g), "d"(c), "l"(v) : "memory");
+        red_fixed(J + g, v, top);
     }
 }
 

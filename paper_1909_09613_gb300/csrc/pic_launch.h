@@ -4,9 +4,7 @@
 
 namespace pic {
 
-bool build_ttable(int l, int scheme, double dtt, TTable *t);
-// the fixed-point form of a table (2D FP64 form), in place of its FP64 coefficients
-void fix_ttable(int l, int scheme, double dtt, TTable *t);
+bool build_ttable(int l, int scheme, double dtt, TTable *t, bool fixed = false);
 int ttable_eval_host(const TTable *t, int l, double delta, double *w);
 
 // CTAs per tile of a single run's 2D particle pass (tile_2d's split), from the tile and particle

@@ -131,8 +131,29 @@ static ld breakpoint(int scheme, ld dtt)
     return f > 1e-15 && f < 1 - 1e-15 ? f : 0;
 }
 
-// Build the table of one axis.  scheme 1 = WT (T_l), 0 = MC (W_l at integer nodes).
-bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
+// The fixed-point form of a table (the FP64 form of a run) from its Taylor coefficients.
+static void fix_table(int l, ld R, ld phib, const ld (*c)[PIC_TK_MAX][5], TTable *t)
+{
+    t->fx.rfrac = (uint64_t)std::ldexp(R - t->Rint, 64);
+    t->fx.phib = (uint64_t)std::ldexp(phib, 64);
+    for (int p = 0; p < 2; ++p) {
+        const ld h = p ? 1 - phib : (phib > 0 ? phib : 1);
+        // 2^shift <= 1 / h < 2^(shift + 1)
+        int sh = 0;
+        while (sh < 62 && std::ldexp(h, sh + 1) <= 1) ++sh;
+        t->fx.shift[p] = sh;
+        t->fx.invm1[p] = (uint64_t)std::ldexp(1 / std::ldexp(h, sh) - 1, 62);
+        for (int k = 0; k < t->K; ++k) {
+            ld hm = 1;
+            for (int m = 0; m <= l; ++m, hm *= h)
+                t->ci[p][k][m] = (int64_t)std::llround(std::ldexp(c[p][k][m] * hm, 59));
+        }
+    }
+}
+
+// Build the table of one axis.  scheme 1 = WT (T_l), 0 = MC (W_l at integer nodes); fixed: the
+// fixed-point form in place of the FP64 and FP32 coefficients.
+bool build_ttable(int l, int scheme, double dtt_d, TTable *t, bool fixed)
 {
     std::memset(t, 0, sizeof(*t));
     if (l < 1 || l > 4) return false;
@@ -153,6 +174,14 @@ bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
     t->phib = (double)phib;
     ld c[2][PIC_TK_MAX][5];
     taylor_coefs(l, scheme, dtt, R, phib, K, c);
+    t->Rfrac_f = (float)t->Rfrac;
+    t->phib_f = (float)t->phib;
+    // the float split must reproduce the same breakpoint ordering
+    if (t->Rfrac_f >= 1.0f) return false;
+    if (fixed) {
+        fix_table(l, R, phib, c, t);
+        return true;
+    }
     for (int p = 0; p < 2; ++p)
         for (int k = 0; k < K; ++k)
             for (int m = 0; m <= l; ++m) t->coef[p][k][m] = (double)c[p][k][m];
@@ -166,38 +195,7 @@ bool build_ttable(int l, int scheme, double dtt_d, TTable *t)
                 }
                 t->cf4[p][m][g] = make_float4(v[0], v[1], v[2], v[3]);
             }
-    t->Rfrac_f = (float)t->Rfrac;
-    t->phib_f = (float)t->phib;
-    // the float split must reproduce the same breakpoint ordering
-    if (t->Rfrac_f >= 1.0f) return false;
     return true;
-}
-
-// The fixed-point form of a table (2D FP64 form), in place of its FP64 coefficients; scheme and
-// dtt as build_ttable had them.
-void fix_ttable(int l, int scheme, double dtt, TTable *t)
-{
-    const ld R = scheme == 1 ? (ld)l / 2 + (ld)dtt : (ld)(l + 1) / 2;
-    const ld phib = breakpoint(scheme, dtt);
-    ld c[2][PIC_TK_MAX][5];
-    taylor_coefs(l, scheme, dtt, R, phib, t->K, c);
-    std::memset(&t->fx, 0, sizeof(t->cf4));
-    std::memset(t->ci, 0, sizeof(t->ci));
-    t->fx.rfrac = (uint64_t)std::ldexp(R - t->Rint, 64);
-    t->fx.phib = (uint64_t)std::ldexp(phib, 64);
-    for (int p = 0; p < 2; ++p) {
-        const ld h = p ? 1 - phib : (phib > 0 ? phib : 1);
-        // 2^shift <= 1 / h < 2^(shift + 1)
-        int sh = 0;
-        while (sh < 62 && std::ldexp(h, sh + 1) <= 1) ++sh;
-        t->fx.shift[p] = sh;
-        t->fx.invm1[p] = (uint64_t)std::ldexp(1 / std::ldexp(h, sh) - 1, 62);
-        for (int k = 0; k < t->K; ++k) {
-            ld hm = 1;
-            for (int m = 0; m <= l; ++m, hm *= h)
-                t->ci[p][k][m] = (int64_t)std::llround(std::ldexp(c[p][k][m] * hm, 59));
-        }
-    }
 }
 
 // Host evaluation of a table (same arithmetic as the device code, in double).
