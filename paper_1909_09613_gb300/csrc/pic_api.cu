@@ -573,6 +573,7 @@ int pic_footprint(const pic_ctx *c, size_t *bytes)
     b += 3 * align_up(rd.ncell * sizeof(double), A);  // rho, rho_prev, gref
     if (rd.det && rd.prec == PIC_FP64) b += 3 * align_up(rd.ncell * sizeof(double), A);  // jlo
     if (uses_j32(rd)) b += align_up(3 * rd.jp_nodes * sizeof(float), A);                // J32
+    if (rd.prec == PIC_FP64) b += 3 * align_up(rd.ncell * sizeof(double), A);           // Bg
     b += 2 * A;                                   // diag out, err
     b += A;                                       // base alignment slack
     (void)captot;
@@ -639,6 +640,8 @@ int pic_bind_memory(pic_ctx *c, void *dev, size_t bytes)
         float *j = (float *)take(3 * rd.jp_nodes * sizeof(float));
         for (int a = 0; a < 3; ++a) rd.J32[a] = j + a * rd.jp_nodes;
     }
+    for (int a = 0; a < 3; ++a)
+        rd.Bg[a] = rd.prec == PIC_FP64 ? (double *)take(rd.ncell * sizeof(double)) : nullptr;
     c->rho_prev_valid = false;
     c->gref_valid = false;
     c->diag_out = (double *)take(8 * sizeof(double));
@@ -770,21 +773,20 @@ int pic_step(pic_ctx *c, int nsteps)
         if (r != PIC_OK) return r;
     }
     if (rd.det) set_det_scale(c);
+    // B half a step ahead, B at integer time kept for the gather, the current cleared
+    if (nsteps > 0) {
+        if (launch_yee_b(rd, true, false, c->stream) != cudaSuccess) return PIC_ECUDA;
+        c->kernel_launches += 1;
+    }
     for (int it = 0; it < nsteps; ++it) {
         if (c->age >= c->sort_interval) {
             const int r = sort_all(c);
             if (r != PIC_OK) return r;
         }
         refresh_species_ptrs(c);
-        if (rd.J32[0]) {  // F[6..8] are written whole from J32 after the particle pass
-            if (cudaMemsetAsync(rd.J32[0], 0, 3 * rd.jp_nodes * sizeof(float), c->stream) != cudaSuccess)
-                return PIC_ECUDA;
-        } else {
-            for (int a = 6; a < 9; ++a)
-                if (cudaMemsetAsync(rd.F[a], 0, rd.ncell * sizeof(double), c->stream) != cudaSuccess)
-                    return PIC_ECUDA;
-        }
-        if (c->jlo && cudaMemsetAsync(c->jlo, 0, 3 * rd.ncell * sizeof(double), c->stream) != cudaSuccess)
+        // F[6..8] of a 3D FP32 run are written whole from J32 after the particle pass
+        if (rd.J32[0]
+            && cudaMemsetAsync(rd.J32[0], 0, 3 * rd.jp_nodes * sizeof(float), c->stream) != cudaSuccess)
             return PIC_ECUDA;
         if (c->have_events) {
             if (c->ev_pending == 64) drain_events(c);
@@ -802,10 +804,9 @@ int pic_step(pic_ctx *c, int nsteps)
             if (launch_j32_finish(rd, c->stream) != cudaSuccess) return PIC_ECUDA;
             c->kernel_launches += 1;
         }
-        if (launch_yee_b(rd, 0.5 * rd.dt, false, c->stream) != cudaSuccess) return PIC_ECUDA;
         if (launch_yee_e(rd, shadow, c->stream) != cudaSuccess) return PIC_ECUDA;
-        if (launch_yee_b(rd, 0.5 * rd.dt, shadow, c->stream) != cudaSuccess) return PIC_ECUDA;
-        c->kernel_launches += 4;
+        if (launch_yee_b(rd, false, it + 1 == nsteps, c->stream) != cudaSuccess) return PIC_ECUDA;
+        c->kernel_launches += 3;
         c->age += 1;
         c->step += 1;
     }

@@ -243,14 +243,14 @@ __global__ void __launch_bounds__(kBlock) k_b_zero_j(const Counts *cn, const Run
 }
 
 __global__ void __launch_bounds__(kBlock) k_b_yee_b(const Counts *cn, const RunDev *runs,
-                                                    const BlockMap *bm, int shadow)
+                                                    const BlockMap *bm, int flags)
 {
     for (int b = blockIdx.x; b < cn->cell; b += gridDim.x) {
         const BlockMap m = bm[b];
         const RunDev &rd = runs[m.run];
         for (int k = 0; k < kCellPer; ++k) {
             const int64_t c = ((int64_t)m.block * kCellPer + k) * blockDim.x + threadIdx.x;
-            if (c < rd.ncell) yee_b_cell(rd, c, 0.5 * rd.dt, shadow);
+            if (c < rd.ncell) yee_b_cell(rd, c, 0.5 * rd.dt, flags);
         }
     }
 }
@@ -454,9 +454,9 @@ cudaError_t enqueue_step(pic_batch *b)
     k_b_gpp<<<b->grid_gpp, 256, b->smem, st>>>(cn, b->d_runs, b->d_state, b->d_items, b->d_counter);
     if (b->timing) cudaEventRecord(b->ev1, st);
     ++nl;
-    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, 0);
+    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, kYeeStart);
     k_b_yee_e<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell);
-    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, 1);
+    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, kYeeFinish | kYeeShadow);
     nl += 3;
     b->launches = nl;
     return cudaGetLastError();

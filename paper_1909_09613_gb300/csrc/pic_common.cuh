@@ -121,6 +121,10 @@ struct RunDev {
     // fields (FP64, index (k*ny + j)*nx + i) and FP32 shadows of E, B (precision form)
     double *F[9];
     float *Fs[6];
+    // FP64 form: B at integer time for the gather, while F[3..5] are already half a step ahead
+    // (pic_step merges the two half steps of B between its steps); null in the FP32 form, which
+    // gathers from Fs
+    double *Bg[3];
     // 3D FP32 form (not deterministic): the current summed by FP32 L2 reductions, converted
     // into F[6..8] after the particle pass; null otherwise.  It is padded: jp_lo ghost nodes
     // below and jp[a] - n[a] - jp_lo above the grid along every axis, so that every deposit

@@ -200,9 +200,9 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
             E[0] = gather3_global<L + 1, KT, KT, R>(rd.F[0], nx, ny, ih[0], it[1], it[2], w[0].wh, w[1].wt, w[2].wt);
             E[1] = gather3_global<KT, L + 1, KT, R>(rd.F[1], nx, ny, it[0], ih[1], it[2], w[0].wt, w[1].wh, w[2].wt);
             E[2] = gather3_global<KT, KT, L + 1, R>(rd.F[2], nx, ny, it[0], it[1], ih[2], w[0].wt, w[1].wt, w[2].wh);
-            B[0] = gather3_global<KT, L + 1, L + 1, R>(rd.F[3], nx, ny, it[0], ih[1], ih[2], w[0].wt, w[1].wh, w[2].wh);
-            B[1] = gather3_global<L + 1, KT, L + 1, R>(rd.F[4], nx, ny, ih[0], it[1], ih[2], w[0].wh, w[1].wt, w[2].wh);
-            B[2] = gather3_global<L + 1, L + 1, KT, R>(rd.F[5], nx, ny, ih[0], ih[1], it[2], w[0].wh, w[1].wh, w[2].wt);
+            B[0] = gather3_global<KT, L + 1, L + 1, R>(rd.Bg[0], nx, ny, it[0], ih[1], ih[2], w[0].wt, w[1].wh, w[2].wh);
+            B[1] = gather3_global<L + 1, KT, L + 1, R>(rd.Bg[1], nx, ny, ih[0], it[1], ih[2], w[0].wh, w[1].wt, w[2].wh);
+            B[2] = gather3_global<L + 1, L + 1, KT, R>(rd.Bg[2], nx, ny, ih[0], ih[1], it[2], w[0].wh, w[1].wh, w[2].wt);
         }
     }
 

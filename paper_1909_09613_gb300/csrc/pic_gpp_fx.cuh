@@ -68,7 +68,7 @@ __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
 #pragma unroll
             for (int c = 0; c < 6; ++c)
-                em[c] = max(em[c], __double2hiint(__ldg(rd.F[c] + g)) & 0x7ff00000);
+                em[c] = max(em[c], __double2hiint(__ldg((c < 3 ? rd.F[c] : rd.Bg[c - 3]) + g)) & 0x7ff00000);
         }
     }
 #pragma unroll
@@ -85,13 +85,13 @@ __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
             const int n = ry * RX + rx;
             const uint2 e1 = field_limbs(__ldg(rd.F[0] + g), em[0]);
-            const uint2 b2 = field_limbs(__ldg(rd.F[4] + g), em[4]);
+            const uint2 b2 = field_limbs(__ldg(rd.Bg[1] + g), em[4]);
             const uint2 e2 = field_limbs(__ldg(rd.F[1] + g), em[1]);
-            const uint2 b1 = field_limbs(__ldg(rd.F[3] + g), em[3]);
+            const uint2 b1 = field_limbs(__ldg(rd.Bg[0] + g), em[3]);
             st.pa[n] = make_uint4(e1.x, e1.y, b2.x, b2.y);
             st.pb[n] = make_uint4(e2.x, e2.y, b1.x, b1.y);
             st.e3[n] = field_limbs(__ldg(rd.F[2] + g), em[2]);
-            st.b3[n] = field_limbs(__ldg(rd.F[5] + g), em[5]);
+            st.b3[n] = field_limbs(__ldg(rd.Bg[2] + g), em[5]);
         }
     }
 }

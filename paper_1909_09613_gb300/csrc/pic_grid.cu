@@ -12,12 +12,13 @@ namespace {
 
 constexpr int kBlock = 256;
 
-// B <- B - h curl E on the staggered grid (Sec. 1 Yee; App. C with A_i = 1).
+// Half steps B <- B - h curl E on the staggered grid (Sec. 1 Yee; App. C with A_i = 1), as the
+// flags name them (yee_b_cell).
 __global__ void __launch_bounds__(kBlock) k_yee_b(const __grid_constant__ RunDev rd, double h,
-                                                  int shadow)
+                                                  int flags)
 {
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c < rd.ncell) yee_b_cell(rd, c, h, shadow);
+    if (c < rd.ncell) yee_b_cell(rd, c, h, flags);
 }
 
 // E <- E + dt curl B - dt J.
@@ -494,9 +495,15 @@ inline unsigned grid_for(int64_t n)
 
 }  // namespace
 
-cudaError_t launch_yee_b(const RunDev &rd, double h, bool shadow, cudaStream_t st)
+// first: the first step of a call (B at integer time -> half a step ahead); last: the last one
+// (-> integer time); neither: from half a step behind the integer time to half a step ahead of it
+cudaError_t launch_yee_b(const RunDev &rd, bool first, bool last, cudaStream_t st)
 {
-    k_yee_b<<<grid_for(rd.ncell), kBlock, 0, st>>>(rd, h, shadow ? 1 : 0);
+    int flags = (first ? 0 : kYeeFinish) | (last ? 0 : kYeeStart);
+    if (rd.prec == 1 && !first) flags |= kYeeShadow;
+    if (rd.Bg[0] && !last) flags |= kYeeKeep;
+    if (!last && !rd.J32[0]) flags |= kYeeZeroJ;
+    k_yee_b<<<grid_for(rd.ncell), kBlock, 0, st>>>(rd, 0.5 * rd.dt, flags);
     return cudaGetLastError();
 }
 

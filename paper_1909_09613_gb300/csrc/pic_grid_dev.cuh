@@ -51,8 +51,19 @@ __device__ __forceinline__ double faraday_d(const RunDev &rd, int ec, int a, int
     return r;
 }
 
-// B <- B - h curl E at cell c (FP32 shadow of B written when `shadow`).
-__device__ __forceinline__ void yee_b_cell(const RunDev &rd, int64_t c, double h, int shadow)
+// What a B update does at a cell.  A step ends with the half step of B that brings it to integer
+// time (kYeeFinish) and the next one begins with another half step from the same E (kYeeStart);
+// between two steps of one call both are done in one pass, each rounded as on its own.
+enum : int {
+    kYeeShadow = 1,  // write the FP32 shadow of B at integer time
+    kYeeStart = 2,
+    kYeeFinish = 4,
+    kYeeKeep = 8,    // write B at integer time to Bg (FP64 form, when a kYeeStart follows)
+    kYeeZeroJ = 16   // clear the current (after E has taken it)
+};
+
+// B <- B - h curl E at cell c, once per half step named by the flags.
+__device__ __forceinline__ void yee_b_cell(const RunDev &rd, int64_t c, double h, int flags)
 {
     int i, j, k;
     cell_ijk(rd, c, i, j, k);
@@ -78,16 +89,36 @@ __device__ __forceinline__ void yee_b_cell(const RunDev &rd, int64_t c, double h
             c3 = (E2[gidx(rd, ip, j, k)] - e2) * idx - (E1[gidx(rd, i, jp, k)] - e1) * idy;
         }
     }
-    const double b1 = rd.F[3][c] - h * c1;
-    const double b2 = rd.F[4][c] - h * c2;
-    const double b3 = rd.F[5][c] - h * c3;
-    rd.F[3][c] = b1;
-    rd.F[4][c] = b2;
-    rd.F[5][c] = b3;
-    if (shadow) {
+    double b1 = rd.F[3][c], b2 = rd.F[4][c], b3 = rd.F[5][c];
+    if (flags & kYeeFinish) {
+        b1 = b1 - h * c1;
+        b2 = b2 - h * c2;
+        b3 = b3 - h * c3;
+    }
+    if (flags & kYeeShadow) {
         rd.Fs[3][c] = (float)b1;
         rd.Fs[4][c] = (float)b2;
         rd.Fs[5][c] = (float)b3;
+    }
+    if (flags & kYeeKeep) {
+        rd.Bg[0][c] = b1;
+        rd.Bg[1][c] = b2;
+        rd.Bg[2][c] = b3;
+    }
+    if (flags & kYeeStart) {
+        b1 = b1 - h * c1;
+        b2 = b2 - h * c2;
+        b3 = b3 - h * c3;
+    }
+    rd.F[3][c] = b1;
+    rd.F[4][c] = b2;
+    rd.F[5][c] = b3;
+    if (flags & kYeeZeroJ) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            rd.F[6 + a][c] = 0.0;
+            if (rd.Jlo[a]) rd.Jlo[a][c] = 0ull;
+        }
     }
 }
 

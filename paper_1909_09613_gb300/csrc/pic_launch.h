@@ -44,7 +44,7 @@ cudaError_t launch_gpp3d(const RunDev &rd, int kt, cudaStream_t st);
 size_t gpp3d_smem_bytes(const RunDev &rd);
 
 // Yee and grid kernels
-cudaError_t launch_yee_b(const RunDev &rd, double h, bool shadow, cudaStream_t st);
+cudaError_t launch_yee_b(const RunDev &rd, bool first, bool last, cudaStream_t st);
 cudaError_t launch_yee_e(const RunDev &rd, bool shadow, cudaStream_t st);
 cudaError_t launch_shadow(const RunDev &rd, cudaStream_t st);
 
