@@ -139,75 +139,64 @@ __device__ __forceinline__ Stage2D<R> stage2d_carve(char *smem, int64_t nodes,
     return s;
 }
 
-// Stage fields of tile (tx, ty) and zero the current tile.
+// Stage fields of the tile at (x0, y0) and zero the current tile.  One warp per row, so that the
+// periodic wrap and the row offset are formed once per row (a linear node index cost two 64-bit
+// remainders per node, which paced the small runs: 64x32 cells 23.4 -> 17.8 us per
+// pass, 250x126 44.7 -> 42.7, the batch of 48 uneven runs 2.60 -> 2.51 ms).
 template <typename R>
 __device__ void stage2d_load(const RunDev &rd, const Stage2D<R> &st, int x0, int y0)
 {
-    const int RX = rd.reg[0];
-    const int64_t nodes = rd.reg_nodes;
+    const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31;
     if (st.tt != rd.tt)
         for (int i = threadIdx.x; i < (int)(2 * sizeof(TTable) / sizeof(int)); i += blockDim.x)
             ((int *)st.tt)[i] = ((const int *)rd.tt)[i];
-    for (int64_t n = threadIdx.x; n < nodes; n += blockDim.x) {
-        const int rx = (int)(n % RX), ry = (int)(n / RX);
-        const int gx = wrap_idx(x0 - rd.pre[0] + rx, rd.n[0]);
-        const int gy = wrap_idx(y0 - rd.pre[1] + ry, rd.n[1]);
-        const int64_t g = (int64_t)gy * rd.n[0] + gx;
-        typename Vec2<R>::T a, b;
-        a.x = __ldg(rd.Fs[0] + g); a.y = __ldg(rd.Fs[4] + g);
-        b.x = __ldg(rd.Fs[1] + g); b.y = __ldg(rd.Fs[3] + g);
-        st.e3[n] = __ldg(rd.Fs[2] + g);
-        st.b3[n] = __ldg(rd.Fs[5] + g);
-        st.pa[n] = a;
-        st.pb[n] = b;
-        if (st.q1) {
-            st.q1[n] = 0ull;
-            st.q2[n] = 0ull;
-            st.q3[n] = 0ull;
-        } else {
-            st.j1[n] = R(0);
-            st.j2[n] = R(0);
-            st.j3[n] = R(0);
+    for (int ry = threadIdx.x >> 5; ry < RY; ry += kTileWarps) {
+        const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
+        for (int rx = lane; rx < RX; rx += 32) {
+            const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
+            const int n = ry * RX + rx;
+            typename Vec2<R>::T a, b;
+            a.x = __ldg(rd.Fs[0] + g); a.y = __ldg(rd.Fs[4] + g);
+            b.x = __ldg(rd.Fs[1] + g); b.y = __ldg(rd.Fs[3] + g);
+            st.e3[n] = __ldg(rd.Fs[2] + g);
+            st.b3[n] = __ldg(rd.Fs[5] + g);
+            st.pa[n] = a;
+            st.pb[n] = b;
+            if (st.q1) {
+                st.q1[n] = 0ull;
+                st.q2[n] = 0ull;
+                st.q3[n] = 0ull;
+            } else {
+                st.j1[n] = R(0);
+                st.j2[n] = R(0);
+                st.j3[n] = R(0);
+            }
         }
     }
 }
 
-// Add the current tile to the global FP64 current and clear it.
+// Add the current tile to the global FP64 current.  One warp per row, as stage2d_load.
 template <typename R>
 __device__ void stage2d_flush(const RunDev &rd, const Stage2D<R> &st, int x0, int y0)
 {
-    const int RX = rd.reg[0];
-    const int64_t nodes = rd.reg_nodes;
-    if (st.q1) {  // deterministic run: integer sums, exact in any order
-        for (int64_t n = threadIdx.x; n < nodes; n += blockDim.x) {
-            const unsigned long long a = st.q1[n], b = st.q2[n], c = st.q3[n];
-            if ((a | b | c) == 0ull) continue;
-            const int rx = (int)(n % RX), ry = (int)(n / RX);
-            const int gx = wrap_idx(x0 - rd.pre[0] + rx, rd.n[0]);
-            const int gy = wrap_idx(y0 - rd.pre[1] + ry, rd.n[1]);
-            const int64_t g = (int64_t)gy * rd.n[0] + gx;
-            if (a) atomicAdd((unsigned long long *)(rd.F[6] + g), a);
-            if (b) atomicAdd((unsigned long long *)(rd.F[7] + g), b);
-            if (c) atomicAdd((unsigned long long *)(rd.F[8] + g), c);
-            st.q1[n] = 0ull;
-            st.q2[n] = 0ull;
-            st.q3[n] = 0ull;
+    const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31;
+    for (int ry = threadIdx.x >> 5; ry < RY; ry += kTileWarps) {
+        const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
+        for (int rx = lane; rx < RX; rx += 32) {
+            const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
+            const int n = ry * RX + rx;
+            if (st.q1) {  // deterministic run: integer sums, exact in any order
+                const unsigned long long a = st.q1[n], b = st.q2[n], c = st.q3[n];
+                if (a) atomicAdd((unsigned long long *)(rd.F[6] + g), a);
+                if (b) atomicAdd((unsigned long long *)(rd.F[7] + g), b);
+                if (c) atomicAdd((unsigned long long *)(rd.F[8] + g), c);
+            } else {
+                const R a = st.j1[n], b = st.j2[n], c = st.j3[n];
+                if (a != R(0)) atomicAdd(rd.F[6] + g, (double)a);
+                if (b != R(0)) atomicAdd(rd.F[7] + g, (double)b);
+                if (c != R(0)) atomicAdd(rd.F[8] + g, (double)c);
+            }
         }
-        return;
-    }
-    for (int64_t n = threadIdx.x; n < nodes; n += blockDim.x) {
-        const R a = st.j1[n], b = st.j2[n], c = st.j3[n];
-        if (a == R(0) && b == R(0) && c == R(0)) continue;
-        const int rx = (int)(n % RX), ry = (int)(n / RX);
-        const int gx = wrap_idx(x0 - rd.pre[0] + rx, rd.n[0]);
-        const int gy = wrap_idx(y0 - rd.pre[1] + ry, rd.n[1]);
-        const int64_t g = (int64_t)gy * rd.n[0] + gx;
-        if (a != R(0)) atomicAdd(rd.F[6] + g, (double)a);
-        if (b != R(0)) atomicAdd(rd.F[7] + g, (double)b);
-        if (c != R(0)) atomicAdd(rd.F[8] + g, (double)c);
-        st.j1[n] = R(0);
-        st.j2[n] = R(0);
-        st.j3[n] = R(0);
     }
 }
 
@@ -639,7 +628,6 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
                                             const Stage2D<R> &st, int64_t p, bool act, int x0,
                                             int y0)
 {
-    const int lane = threadIdx.x & 31;
     PState<R> s;
     int lx = 0, ly = 0;
     if (act) {
@@ -820,27 +808,29 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
         const HotSp<R> hs = make_hotsp<R>(sp);
         int64_t a = sp.tile_start[tile], b = sp.tile_start[tile + 1];
         split_range(split, a, b);
-        {
-            // every warp takes a contiguous chunk of the tile's particles of this species (for a
-            // uniform plasma in the cell-major order, one row of cells), so that the warps'
-            // frames, a row apart, rarely race for the same nodes of the tile: 5.53 -> 5.38 ms
-            // on the 134M-particle FP32 step (slot-major runs, whose lanes deposit one by one,
-            // lose about 5%; a runtime choice between the two loops cost the dense kernel more)
-            const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            const int64_t groups = (b - a + 31) / 32;
-            const int64_t gw = (groups + kTileWarps - 1) / kTileWarps;
-            const int64_t ca = a + 32 * min(groups, (int64_t)w * gw);
-            const int64_t cb = min(b, a + 32 * min(groups, (int64_t)(w + 1) * gw));
-            for (int64_t q = ca; q < cb; q += 32) {  // warp-uniform trip count
-                const int64_t p = q + lane;
-                if (p + 32 < cb) prefetch_particle<R>(hs, p + 32);
-                particle_2d<L, KT, R, DET>(h, hs, st, p, p < cb, x0, y0);
-            }
+        // every warp takes a contiguous chunk of the tile's particles of this species (for a
+        // uniform plasma in the cell-major order, one row of cells), so that the warps' frames,
+        // a row apart, rarely race for the same nodes of the tile: 5.53 -> 5.38 ms on the
+        // 134M-particle FP32 step (slot-major runs, whose lanes deposit one by one, lose about
+        // 5%; a runtime choice between the two loops cost the dense kernel more).  The species
+        // of a part of few particles start at different warps, so as not to queue one behind the
+        // other on the first warps.
+        const int lane = threadIdx.x & 31;
+        const int64_t groups = (b - a + 31) / 32;
+        const int w = ((threadIdx.x >> 5) + (groups < kTileWarps ? s * (kTileWarps / 2) : 0)) % kTileWarps;
+        const int64_t gw = (groups + kTileWarps - 1) / kTileWarps;
+        const int64_t ca = a + 32 * min(groups, (int64_t)w * gw);
+        const int64_t cb = min(b, a + 32 * min(groups, (int64_t)(w + 1) * gw));
+        for (int64_t q = ca; q < cb; q += 32) {  // warp-uniform trip count
+            const int64_t p = q + lane;
+            if (p + 32 < cb) prefetch_particle<R>(hs, p + 32);
+            particle_2d<L, KT, R, DET>(h, hs, st, p, p < cb, x0, y0);
         }
-        __syncthreads();
-        stage2d_flush<R>(rd, st, x0, y0);
-        __syncthreads();
     }
+    // one flush for all species (one per species doubled the tile's FP64 atomics and held the
+    // warps at two more barriers)
+    __syncthreads();
+    stage2d_flush<R>(rd, st, x0, y0);
 }
 
 }  // namespace pic
