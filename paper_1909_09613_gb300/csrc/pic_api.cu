@@ -453,7 +453,7 @@ int pic_create(const int32_t grid[3], const double dx[3], double dt, int spline_
     c->kt = 0;
     for (int a = 0; a < 3; ++a) {
         if (a >= dim) { build_ttable(spline_order, PIC_SCHEME_MC, 0.5, &rd.tt[a]); continue; }
-        if (!build_ttable(spline_order, scheme, rd.dtt[a], &rd.tt[a], dim == 2 && rd.prec == PIC_FP64)) {
+        if (!build_ttable(spline_order, scheme, rd.dtt[a], &rd.tt[a], rd.prec == PIC_FP64)) {
             delete c;
             return PIC_ECFL;
         }

@@ -1,5 +1,5 @@
 // Instantiations of the fused particle pass in 3D, both forms.
-#include "pic_gpp3d.cuh"
+#include "pic_gpp3d_fx.cuh"
 #include "pic_launch.h"
 
 namespace pic {
@@ -12,13 +12,30 @@ template <int L, int KT>
 __global__ void __launch_bounds__(128, (L <= 2 ? 4 : 1)) k_gpp3d_f32(const __grid_constant__ RunDev rd)
 {
     extern __shared__ __align__(16) float sf3[];
-    tile_3d<L, KT, float>(rd, blockIdx.x, sf3);
+    tile_3d<L, KT>(rd, blockIdx.x, sf3);
 }
 
-template <int L, int KT>
-__global__ void __launch_bounds__(128) k_gpp3d_f64(const __grid_constant__ RunDev rd)
+template <int L, int KT, bool DET>
+__global__ void __launch_bounds__(128, L <= 2 ? 4 : 2) k_gpp3d_f64(const __grid_constant__ RunDev rd)
 {
-    tile_3d<L, KT, double>(rd, blockIdx.x);
+    tile3_fx<L, KT, DET>(rd, blockIdx.x);
+}
+
+// CTAs per tile of the FP64 form, which stages nothing and so splits its tiles freely: eight
+// waves of four CTAs per SM, so that the last wave is short, while every part keeps a particle of
+// a species per thread.
+unsigned tile_parts3(const RunDev &rd)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess
+        || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    int64_t n = 0;
+    for (int s = 0; s < rd.nsp; ++s) n = rd.sp[s].n > n ? rd.sp[s].n : n;
+    const int64_t most = (n / rd.ntiles + 127) / 128;
+    const int64_t want = (8 * 4 * (int64_t)sms + rd.ntiles - 1) / rd.ntiles;
+    const int64_t parts = want < most ? want : most;
+    return (unsigned)(parts > 1 ? parts : 1);
 }
 
 template <int L, int KT>
@@ -31,7 +48,9 @@ cudaError_t go(const RunDev &rd, cudaStream_t st)
         if (e != cudaSuccess) return e;
         k_gpp3d_f32<L, KT><<<(unsigned)rd.ntiles, 128, smem, st>>>(rd);
     } else {
-        k_gpp3d_f64<L, KT><<<(unsigned)rd.ntiles, 128, 0, st>>>(rd);
+        const dim3 grid((unsigned)rd.ntiles, tile_parts3(rd));
+        if (rd.det) k_gpp3d_f64<L, KT, true><<<grid, 128, 0, st>>>(rd);
+        else k_gpp3d_f64<L, KT, false><<<grid, 128, 0, st>>>(rd);
     }
     return cudaGetLastError();
 }

@@ -1,6 +1,5 @@
-// Tile kernel of the fused particle pass in 3D: the FP32 form stages the tile's fields in
-// shared memory, the FP64 form reads them through L1; both add the current by global
-// reductions.
+// Tile kernel of the fused particle pass in 3D, FP32 form: the tile's fields staged in shared
+// memory, the current added by global reductions (FP64 form: pic_gpp3d_fx.cuh).
 #pragma once
 #include "pic_gpp_kernels.cuh"
 
@@ -28,48 +27,35 @@ __device__ inline void stage3d_load(const RunDev &rd, float *sf, int x0, int y0,
     }
 }
 
-// The stored state of one particle as loaded (FP32 form: cell index, offsets, momenta; FP64
-// form: positions in cell units, momenta).
-template <typename R>
+// The stored state of one particle as loaded: cell index, offsets, momenta.
 struct Raw3 {
     int cell;
-    R x[3];
-    R u[3];
+    float x[3];
+    float u[3];
 };
 
-template <typename R>
-__device__ __forceinline__ void load_raw3(const SpeciesDev &sp, int64_t p, Raw3<R> &r)
+__device__ __forceinline__ void load_raw3(const SpeciesDev &sp, int64_t p, Raw3 &r)
 {
-    if constexpr (sizeof(R) == 4) r.cell = __ldg(sp.cell + p);
-    else r.cell = 0;
+    r.cell = __ldg(sp.cell + p);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        r.x[a] = __ldg((const R *)sp.pos[a] + p);
-        r.u[a] = __ldg((const R *)sp.mom[a] + p);
+        r.x[a] = __ldg((const float *)sp.pos[a] + p);
+        r.u[a] = __ldg((const float *)sp.mom[a] + p);
     }
 }
 
-template <typename R>
-__device__ __forceinline__ void decode_raw3(const RunDev &rd, const Raw3<R> &r, PState<R> &s)
+__device__ __forceinline__ void decode_raw3(const RunDev &rd, const Raw3 &r, PState<float> &s)
 {
-    if constexpr (sizeof(R) == 4) {
-        const int nxy = rd.n[0] * rd.n[1];
-        s.c[2] = fast_div(r.cell, rd.div_n01.m, rd.div_n01.s);
-        const int q = r.cell - s.c[2] * nxy;
-        s.c[1] = fast_div(q, rd.div_n0.m, rd.div_n0.s);
-        s.c[0] = q - s.c[1] * rd.n[0];
+    const int nxy = rd.n[0] * rd.n[1];
+    s.c[2] = fast_div(r.cell, rd.div_n01.m, rd.div_n01.s);
+    const int q = r.cell - s.c[2] * nxy;
+    s.c[1] = fast_div(q, rd.div_n0.m, rd.div_n0.s);
+    s.c[0] = q - s.c[1] * rd.n[0];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) s.d[a] = r.x[a];
-    } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const double f = floor(r.x[a]);
-            s.c[a] = min(max((int)f, 0), rd.n[a] - 1);  // a non-finite position stays in range
-            s.d[a] = r.x[a] - f;
-        }
+    for (int a = 0; a < 3; ++a) {
+        s.d[a] = r.x[a];
+        s.u[a] = r.u[a];
     }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) s.u[a] = r.u[a];
 }
 
 // One staggered field component at a particle from the staged tile: sum over the stencil
@@ -97,48 +83,24 @@ __device__ __forceinline__ R gather3_staged(const float *f, int RX, int RXY, int
     return acc;
 }
 
-// The same through L1 from the global field (wrapped node indices per axis).
-template <int NA, int NB, int NC, typename R, typename F>
-__device__ __forceinline__ R gather3_global(const F *f, int64_t nx, int64_t ny, const int *xi,
-                                            const int *yi, const int *zi, const R *wx,
-                                            const R *wy, const R *wz)
-{
-    R acc = R(0);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        R r2 = R(0);
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const int64_t row = ((int64_t)zi[c] * ny + yi[b]) * nx;
-            R r1 = R(0);
-#pragma unroll
-            for (int a = 0; a < NA; ++a) r1 += wx[a] * (R)__ldg(f + row + xi[a]);
-            r2 += wy[b] * r1;
-        }
-        acc += wz[c] * r2;
-    }
-    return acc;
-}
-
-// One particle, 3D: fields from the tile's shared-memory stage (STAGED, FP32 form: sf, tile
-// origin x0, y0, z0) or through L1 (FP64 form), current by global reductions (FP32 form: into
-// the padded FP32 current RunDev::J32, whose windows need no wrapping, so each row of a window
-// is one pointer and its x nodes go in as aligned pairs, red.global.add.v2.f32 -- fewer
-// reduction requests for the L2, which bounds this kernel; FP64 form and deterministic runs:
-// into F[6..8]).  Called by all 32 lanes of a warp together (the window-row skips of the
-// deposit are decided per warp); lanes with act == false carry no particle.  raw: the
-// particle's stored state, loaded by the caller.
-template <int L, int KT, typename R, bool STAGED = false>
+// One particle, 3D: fields from the tile's shared-memory stage (sf, tile origin x0, y0, z0),
+// current by global reductions: into the padded FP32 current RunDev::J32, whose windows need no
+// wrapping, so each row of a window is one pointer and its x nodes go in as aligned pairs,
+// red.global.add.v2.f32 (fewer reduction requests for the L2, which bounds this kernel);
+// deterministic runs: into F[6..8].  Called by all 32 lanes of a warp together (the window-row
+// skips of the deposit are decided per warp); lanes with act == false carry no particle.  raw:
+// the particle's stored state, loaded by the caller.
+template <int L, int KT>
 __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &sp, int64_t p,
-                                            bool act, const Raw3<R> &raw,
-                                            const float *sf = nullptr, int x0 = 0, int y0 = 0,
-                                            int z0 = 0)
+                                            bool act, const Raw3 &raw, const float *sf, int x0,
+                                            int y0, int z0)
 {
+    typedef float R;
     PState<R> s;
-    decode_raw3<R>(rd, raw, s);
+    decode_raw3(rd, raw, s);
     const int nx = rd.n[0], ny = rd.n[1];
     int lc[3] = {0, 0, 0};
-    if constexpr (STAGED) {
+    {
         const int org[3] = {x0, y0, z0};
         bool ok = act;
 #pragma unroll
@@ -166,63 +128,34 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
     // ---- gather (Eq. interpolation-EB-real-mod in 3D):
     // E1: W T T ; E2: T W T ; E3: T T W ; B1: T W W ; B2: W T W ; B3: W W T (x, y, z)
     R E[3], B[3];
-    if constexpr (STAGED) {
-        const int RX = rd.reg[0], RXY = rd.reg[0] * rd.reg[1], nodes = (int)rd.reg_nodes;
-        int h[3], t[3];  // first staged node of the half-integer and integer stencils
+    const int RX = rd.reg[0], RXY = rd.reg[0] * rd.reg[1], nodes = (int)rd.reg_nodes;
+    int h[3], t[3];  // first staged node of the half-integer and integer stencils
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            h[a] = lc[a] + rd.pre[a] + w[a].bh;
-            t[a] = lc[a] + rd.pre[a] + w[a].bt;
-        }
-        E[0] = gather3_staged<L + 1, KT, KT, R>(sf, RX, RXY, h[0], t[1], t[2], w[0].wh, w[1].wt, w[2].wt);
-        E[1] = gather3_staged<KT, L + 1, KT, R>(sf + nodes, RX, RXY, t[0], h[1], t[2], w[0].wt, w[1].wh, w[2].wt);
-        E[2] = gather3_staged<KT, KT, L + 1, R>(sf + 2 * nodes, RX, RXY, t[0], t[1], h[2], w[0].wt, w[1].wt, w[2].wh);
-        B[0] = gather3_staged<KT, L + 1, L + 1, R>(sf + 3 * nodes, RX, RXY, t[0], h[1], h[2], w[0].wt, w[1].wh, w[2].wh);
-        B[1] = gather3_staged<L + 1, KT, L + 1, R>(sf + 4 * nodes, RX, RXY, h[0], t[1], h[2], w[0].wh, w[1].wt, w[2].wh);
-        B[2] = gather3_staged<L + 1, L + 1, KT, R>(sf + 5 * nodes, RX, RXY, h[0], h[1], t[2], w[0].wh, w[1].wh, w[2].wt);
-    } else {
-        int ih[3][L + 1], it[3][KT];  // wrapped global node indices
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-#pragma unroll
-            for (int k = 0; k <= L; ++k) ih[a][k] = wrap_idx(s.c[a] + w[a].bh + k, rd.n[a]);
-#pragma unroll
-            for (int k = 0; k < KT; ++k) it[a][k] = wrap_idx(s.c[a] + w[a].bt + k, rd.n[a]);
-        }
-        if constexpr (sizeof(R) == 4) {
-            E[0] = gather3_global<L + 1, KT, KT, R>(rd.Fs[0], nx, ny, ih[0], it[1], it[2], w[0].wh, w[1].wt, w[2].wt);
-            E[1] = gather3_global<KT, L + 1, KT, R>(rd.Fs[1], nx, ny, it[0], ih[1], it[2], w[0].wt, w[1].wh, w[2].wt);
-            E[2] = gather3_global<KT, KT, L + 1, R>(rd.Fs[2], nx, ny, it[0], it[1], ih[2], w[0].wt, w[1].wt, w[2].wh);
-            B[0] = gather3_global<KT, L + 1, L + 1, R>(rd.Fs[3], nx, ny, it[0], ih[1], ih[2], w[0].wt, w[1].wh, w[2].wh);
-            B[1] = gather3_global<L + 1, KT, L + 1, R>(rd.Fs[4], nx, ny, ih[0], it[1], ih[2], w[0].wh, w[1].wt, w[2].wh);
-            B[2] = gather3_global<L + 1, L + 1, KT, R>(rd.Fs[5], nx, ny, ih[0], ih[1], it[2], w[0].wh, w[1].wh, w[2].wt);
-        } else {
-            E[0] = gather3_global<L + 1, KT, KT, R>(rd.F[0], nx, ny, ih[0], it[1], it[2], w[0].wh, w[1].wt, w[2].wt);
-            E[1] = gather3_global<KT, L + 1, KT, R>(rd.F[1], nx, ny, it[0], ih[1], it[2], w[0].wt, w[1].wh, w[2].wt);
-            E[2] = gather3_global<KT, KT, L + 1, R>(rd.F[2], nx, ny, it[0], it[1], ih[2], w[0].wt, w[1].wt, w[2].wh);
-            B[0] = gather3_global<KT, L + 1, L + 1, R>(rd.Bg[0], nx, ny, it[0], ih[1], ih[2], w[0].wt, w[1].wh, w[2].wh);
-            B[1] = gather3_global<L + 1, KT, L + 1, R>(rd.Bg[1], nx, ny, ih[0], it[1], ih[2], w[0].wh, w[1].wt, w[2].wh);
-            B[2] = gather3_global<L + 1, L + 1, KT, R>(rd.Bg[2], nx, ny, ih[0], ih[1], it[2], w[0].wh, w[1].wh, w[2].wt);
-        }
+    for (int a = 0; a < 3; ++a) {
+        h[a] = lc[a] + rd.pre[a] + w[a].bh;
+        t[a] = lc[a] + rd.pre[a] + w[a].bt;
     }
+    E[0] = gather3_staged<L + 1, KT, KT, R>(sf, RX, RXY, h[0], t[1], t[2], w[0].wh, w[1].wt, w[2].wt);
+    E[1] = gather3_staged<KT, L + 1, KT, R>(sf + nodes, RX, RXY, t[0], h[1], t[2], w[0].wt, w[1].wh, w[2].wt);
+    E[2] = gather3_staged<KT, KT, L + 1, R>(sf + 2 * nodes, RX, RXY, t[0], t[1], h[2], w[0].wt, w[1].wt, w[2].wh);
+    B[0] = gather3_staged<KT, L + 1, L + 1, R>(sf + 3 * nodes, RX, RXY, t[0], h[1], h[2], w[0].wt, w[1].wh, w[2].wh);
+    B[1] = gather3_staged<L + 1, KT, L + 1, R>(sf + 4 * nodes, RX, RXY, h[0], t[1], h[2], w[0].wh, w[1].wt, w[2].wh);
+    B[2] = gather3_staged<L + 1, L + 1, KT, R>(sf + 5 * nodes, RX, RXY, h[0], h[1], t[2], w[0].wh, w[1].wh, w[2].wt);
 
     // ---- Boris push and move ----
     const R ig = boris<R>(R(sp.qmdt_half), E, B, s.u);
-    R o[3], dl[3], xs[3];
-    int cn[3], shv[3];
+    R o[3], dl[3], xs;
+    int cn[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         dl[a] = R(rd.dtt[a]) * s.u[a] * ig;
-        shv[a] = move_axis<R>(s.d[a], dl[a], s.c[a], rd.n[a], o[a], cn[a], xs[a]);
+        move_axis<R>(s.d[a], dl[a], s.c[a], rd.n[a], o[a], cn[a], xs);
     }
 
     // ---- Esirkepov deposit ----
     AxisS<L, R> S[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if constexpr (sizeof(R) == 4) axis_shapes_dd<L, true>(s.d[a], dl[a], S[a]);
-        else axis_shapes<L, R>(s.d[a], shv[a], o[a], S[a]);
-    }
+    for (int a = 0; a < 3; ++a) axis_shapes_dd<L, true>(s.d[a], dl[a], S[a]);
     R DS[3][L + 2], P[3][L + 2];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -255,7 +188,7 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
             fc1[a][k] = R(0.5) * S[a].s0[k] + third * DS[a][k];
         }
     }
-    if (sizeof(R) == 4 && !rd.det) {
+    if (!rd.det) {
         // padded FP32 current: the window of axis a starts at c_a + wb_a + jp_lo, unwrapped
         const int PX = rd.jp[0], PXY = rd.jp[0] * rd.jp[1];
         const int w0 = ((s.c[2] + S[2].wb + rd.jp_lo) * rd.jp[1] + (s.c[1] + S[1].wb + rd.jp_lo)) * PX
@@ -338,19 +271,8 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
                         const int g = base + off[ax][ka];
                         const R v = kP[ka] * perp;
                         if (!act || v == R(0)) continue;
-                        if (rd.det) {
-                            if constexpr (sizeof(R) == 4) {
-                                atomicAdd((unsigned long long *)(rd.F[6 + ax] + g),
-                                          det_word32(v, rd.det_inv32));
-                            } else {
-                                unsigned long long hi, lo;
-                                det_words64(v, rd.det_inv64, hi, lo);
-                                atomicAdd((unsigned long long *)(rd.F[6 + ax] + g), hi);
-                                atomicAdd(rd.Jlo[ax] + g, lo);
-                            }
-                        } else {
-                            atomicAdd(rd.F[6 + ax] + g, (double)v);
-                        }
+                        atomicAdd((unsigned long long *)(rd.F[6 + ax] + g),
+                                  det_word32(v, rd.det_inv32));
                     }
                 }
             }
@@ -359,14 +281,9 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
     if (!act) return;
 #pragma unroll
     for (int a = 0; a < 3; ++a) ((R *)sp.mom[a])[p] = s.u[a];
-    if constexpr (sizeof(R) == 4) {
-        sp.cell[p] = (cn[2] * ny + cn[1]) * nx + cn[0];
+    sp.cell[p] = (cn[2] * ny + cn[1]) * nx + cn[0];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) ((float *)sp.pos[a])[p] = o[a];
-    } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) ((double *)sp.pos[a])[p] = xs[a];  // = cn + o
-    }
+    for (int a = 0; a < 3; ++a) ((float *)sp.pos[a])[p] = o[a];
 }
 
 // Ask the memory system for the particle stream of a later iteration, 3D (see
@@ -383,44 +300,35 @@ __device__ __forceinline__ void prefetch_particle_3d(const SpeciesDev &sp, int64
         asm volatile("prefetch.global.L1 [%0];" ::"l"((const char *)sp.cell + p * 4));
 }
 
-// All particles of one 3D tile.  FP32 form: the tile's fields and halo are staged in shared
-// memory first (sf, 6 x reg_nodes floats; the FP32 3D sort interval keeps every particle
-// within one cell of its sorted tile); FP64 form: fields through L1.  A warp's lanes take 32
-// consecutive particles (warp-uniform trip count) and ask for the stream of their next
-// iteration ahead (into L1); the first particles of every species are requested before the
-// stage load.
-template <int L, int KT, typename R>
-__device__ void tile_3d(const RunDev &rd, int64_t tile, float *sf = nullptr)
+// All particles of one 3D tile: the tile's fields and halo are staged in shared memory first
+// (sf, 6 x reg_nodes floats; the FP32 3D sort interval keeps every particle within one cell of
+// its sorted tile).  A warp's lanes take 32 consecutive particles (warp-uniform trip count) and
+// ask for the stream of their next iteration ahead (into L1); the first particles of every
+// species are requested before the stage load.
+template <int L, int KT>
+__device__ void tile_3d(const RunDev &rd, int64_t tile, float *sf)
 {
     const int lane = threadIdx.x & 31;
     for (int s = 0; s < rd.nsp; ++s) {
         const int64_t p = rd.sp[s].tile_start[tile] + threadIdx.x;
-        if (p < rd.sp[s].tile_start[tile + 1]) prefetch_particle_3d<R>(rd.sp[s], p);
+        if (p < rd.sp[s].tile_start[tile + 1]) prefetch_particle_3d<float>(rd.sp[s], p);
     }
-    int x0 = 0, y0 = 0, z0 = 0;
-    if constexpr (sizeof(R) == 4) {
-        const int tx = (int)(tile % rd.ntile[0]);
-        const int ty = (int)((tile / rd.ntile[0]) % rd.ntile[1]);
-        const int tz = (int)(tile / ((int64_t)rd.ntile[0] * rd.ntile[1]));
-        x0 = tx * rd.tile[0];
-        y0 = ty * rd.tile[1];
-        z0 = tz * rd.tile[2];
-        stage3d_load(rd, sf, x0, y0, z0);
-        __syncthreads();
-    }
+    const int tx = (int)(tile % rd.ntile[0]);
+    const int ty = (int)((tile / rd.ntile[0]) % rd.ntile[1]);
+    const int tz = (int)(tile / ((int64_t)rd.ntile[0] * rd.ntile[1]));
+    const int x0 = tx * rd.tile[0], y0 = ty * rd.tile[1], z0 = tz * rd.tile[2];
+    stage3d_load(rd, sf, x0, y0, z0);
+    __syncthreads();
     for (int s = 0; s < rd.nsp; ++s) {
         const SpeciesDev &sp = rd.sp[s];
         const int64_t a = sp.tile_start[tile], b = sp.tile_start[tile + 1];
         for (int64_t q = a + (threadIdx.x & ~31); q < b; q += blockDim.x) {
             const int64_t p = q + lane;
             const bool act = p < b;
-            if (p + blockDim.x < b) prefetch_particle_3d<R>(sp, p + blockDim.x);
-            Raw3<R> cur = {};
-            if (act) load_raw3<R>(sp, p, cur);
-            if constexpr (sizeof(R) == 4)
-                particle_3d<L, KT, R, true>(rd, sp, p, act, cur, sf, x0, y0, z0);
-            else
-                particle_3d<L, KT, R>(rd, sp, p, act, cur);
+            if (p + blockDim.x < b) prefetch_particle_3d<float>(sp, p + blockDim.x);
+            Raw3 cur = {};
+            if (act) load_raw3(sp, p, cur);
+            particle_3d<L, KT>(rd, sp, p, act, cur, sf, x0, y0, z0);
         }
     }
 }
