@@ -140,16 +140,13 @@ int latched_status(pic_ctx *c)
     return PIC_OK;
 }
 
-int sort_species(pic_ctx *c, int s)
+// Sort species s0 .. s0 + ns - 1 by the same launches.
+int sort_species(pic_ctx *c, int s0, int ns)
 {
-    RunDev rd = c->rd;
     refresh_species_ptrs(c);
-    rd = c->rd;
-    cudaError_t e = launch_sort(rd, s, c->tile_start[s], c->bufB[s], c->bufB[s] + 3,
-                                (int32_t *)c->bufB[s][6], c->stream);
-    if (e != cudaSuccess) return PIC_ECUDA;
-    c->kernel_launches += rd.sp[s].n > 0 ? 6 : 3;
-    for (int i = 0; i < 7; ++i) std::swap(c->bufA[s][i], c->bufB[s][i]);
+    if (launch_sort(c->rd, s0, ns, c->stream, &c->kernel_launches) != cudaSuccess) return PIC_ECUDA;
+    for (int s = s0; s < s0 + ns; ++s)
+        for (int i = 0; i < 7; ++i) std::swap(c->bufA[s][i], c->bufB[s][i]);
     refresh_species_ptrs(c);
     return PIC_OK;
 }
@@ -169,8 +166,9 @@ void drain_events(pic_ctx *c)
 
 int sort_all(pic_ctx *c)
 {
-    for (int s = 0; s < c->rd.nsp; ++s) {
-        const int r = sort_species(c, s);
+    const int ns = c->rd.sc_more ? c->rd.nsp : 1;
+    for (int s = 0; s < c->rd.nsp; s += ns) {
+        const int r = sort_species(c, s, ns);
         if (r != PIC_OK) return r;
     }
     c->age = 0;
@@ -202,7 +200,7 @@ int finish_load(pic_ctx *c, int species)
     // the loaded species is sorted now; the shared sort age keeps counting the steps since the
     // other species were sorted (resetting it could let them drift past the staged halo
     // before the next automatic sort)
-    const int r = sort_species(c, species);
+    const int r = sort_species(c, species, 1);
     if (r != PIC_OK) return r;
     c->loaded[species] = true;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return PIC_ECUDA;
@@ -626,6 +624,13 @@ int pic_bind_memory(pic_ctx *c, void *dev, size_t bytes)
     c->sc.tile_count = (int64_t *)take((rd.ntiles + 1) * sizeof(int64_t));
     c->staging_bytes = staging_size(rd, capmax);
     c->staging = take(c->staging_bytes);
+    // the further species' sort scratch lies in the staging buffer, where it fits (up to kChunk
+    // particles of a species): loads and read-backs use it in stream order, never across a sort
+    rd.sc_more = nullptr;
+    rd.sc_cap = capmax;
+    if (rd.nsp > 1
+        && (rd.nsp - 1) * sort_set_bytes(rd.ntiles * TC, rd.ntiles, capmax) <= (int64_t)c->staging_bytes)
+        rd.sc_more = c->staging;
     c->rho = (double *)take(rd.ncell * sizeof(double));
     c->rho_prev = (double *)take(rd.ncell * sizeof(double));
     c->gref = (double *)take(rd.ncell * sizeof(double));

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kBlock) k_b_count(const Counts *cn, const RunD
         for (int64_t e = first_block(d); e < part_blocks(n); e += gridDim.x)
             for (int k = 0; k < kPartPer; ++k) {
                 const int64_t p = (e * kPartPer + k) * blockDim.x + threadIdx.x;
-                if (p < n) sort_count_one(rd, s, p);
+                if (p < n) sort_count_one(rd, rd.sc, s, p);
             }
     }
 }
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kTileThreads) k_b_tile_sum(const Counts *cn, c
     for (int d = 0; d < nd; ++d) {
         const RunDev &rd = runs[due[d]];
         for (int64_t t = first_block(d); t < rd.ntiles; t += gridDim.x) {
-            sort_tile_sum_block(rd, t);
+            sort_tile_sum_block(rd, rd.sc, t);
             __syncthreads();
         }
     }
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kTileThreads) k_b_layout(const Counts *cn, con
     for (int d = 0; d < nd; ++d) {
         const RunDev &rd = runs[due[d]];
         for (int64_t t = first_block(d); t < rd.ntiles; t += gridDim.x) {
-            sort_layout_block(rd, rd.sp[s].tile_start, t);
+            sort_layout_block(rd, rd.sc, rd.sp[s].tile_start[t], t);
             __syncthreads();
         }
     }
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kBlock) k_b_place(const Counts *cn, const RunD
         for (int64_t e = first_block(d); e < part_blocks(n); e += gridDim.x)
             for (int k = 0; k < kPartPer; ++k) {
                 const int64_t p = (e * kPartPer + k) * blockDim.x + threadIdx.x;
-                if (p < n) sort_place_one(rd, p);
+                if (p < n) sort_place_one(rd.sc, p);
             }
     }
 }
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kBlock) k_b_scatter(const Counts *cn, const Ru
         for (int64_t e = first_block(d); e < part_blocks(sp.n); e += gridDim.x)
             for (int k = 0; k < kPartPer; ++k) {
                 const int64_t r = (e * kPartPer + k) * blockDim.x + threadIdx.x;
-                if (r < sp.n) sort_scatter_one(rd, s, r, sp.pos_alt, sp.mom_alt, sp.cell_alt);
+                if (r < sp.n) sort_scatter_one(rd, rd.sc, s, r);
             }
     }
 }

@@ -46,7 +46,7 @@ struct TTable {
     };
 };
 
-// Scratch of the tile sort (one set per run; the species are sorted one after the other).
+// Scratch of the tile sort of one species.
 struct SortScratch {
     int32_t *cnt;         // ntiles * TC
     int32_t *cell_first;  // ntiles * TC
@@ -137,7 +137,11 @@ struct RunDev {
     TTable tt[3];
     int nsp;
     SpeciesDev sp[PIC_NSP_MAX];
+    // sort scratch: sc, and where they fit (sc_more not null) one more set per further species,
+    // so that all species are sorted by the same launches (sort_scratch)
     SortScratch sc;
+    char *sc_more;
+    int64_t sc_cap;  // particles of a set
     int32_t *err;
     // deterministic current (pic_options.deterministic): every contribution is added as a
     // 64-bit fixed-point integer, so the sums do not depend on the order of the atomics.
@@ -150,6 +154,28 @@ struct RunDev {
     double det_scale;
     unsigned long long *Jlo[3];
 };
+
+// Bytes of one further scratch set, and set k (0: the run's own).
+__host__ __device__ inline int64_t sort_set_bytes(int64_t keys, int64_t tiles, int64_t cap)
+{
+    return (8 * (tiles + 1) + 8 * keys + 16 * cap + 255) / 256 * 256;
+}
+
+__host__ __device__ inline SortScratch sort_scratch(const RunDev &rd, int k)
+{
+    if (k == 0) return rd.sc;
+    const int64_t keys = rd.ntiles * rd.tile[0] * rd.tile[1] * rd.tile[2];
+    char *p = rd.sc_more + (k - 1) * sort_set_bytes(keys, rd.ntiles, rd.sc_cap);
+    SortScratch c;
+    c.tile_count = (int64_t *)p;
+    c.cnt = (int32_t *)(c.tile_count + rd.ntiles + 1);
+    c.cell_first = c.cnt + keys;
+    c.slot = c.cell_first + keys;
+    c.key = c.slot + rd.sc_cap;
+    c.idx = c.key + rd.sc_cap;
+    c.pos = c.idx + rd.sc_cap;
+    return c;
+}
 
 // Fixed-point forms of a current contribution v (see RunDev::det).
 __device__ __forceinline__ unsigned long long det_word32(float v, float inv)

@@ -81,8 +81,8 @@ cudaError_t launch_det_finish(const RunDev &rd, cudaStream_t st);
 // FP32 current of a 3D FP32 run (RunDev::J32) -> F[6..8] (after the particle pass)
 cudaError_t launch_j32_finish(const RunDev &rd, cudaStream_t st);
 
-// tile sort of one species
-cudaError_t launch_sort(const RunDev &rd, int s, int64_t *tile_start, void *const *dst_pos,
-                        void *const *dst_mom, int32_t *dst_cell, cudaStream_t st);
+// tile sort of species s0 .. s0 + ns - 1 (ns > 1 only with RunDev::sc_more) into their other
+// buffers; adds its kernels to *launches
+cudaError_t launch_sort(const RunDev &rd, int s0, int ns, cudaStream_t st, int64_t *launches);
 
 }  // namespace pic

@@ -65,13 +65,14 @@ __device__ __forceinline__ int sort_block_excl_scan(int v, int *total)
 // 1. tile-major cell key of particle p, the particle count of every key, and a provisional
 //    place among the particles of its key (taken from an atomic, so not reproducible; stage 5
 //    replaces it by the particle's rank in the previous order)
-__device__ __forceinline__ void sort_count_one(const RunDev &rd, int s, int64_t p)
+__device__ __forceinline__ void sort_count_one(const RunDev &rd, const SortScratch &sc, int s,
+                                               int64_t p)
 {
     const SpeciesDev &sp = rd.sp[s];
     int c[3];
     sort_cell_coords(rd, sp, p, c);
     const int key = sort_tile_major_key(rd, c);
-    rd.sc.key[p] = key;
+    sc.key[p] = key;
     // lanes with the same key (neighbours in a sorted store) take consecutive slots from one
     // atomic of their leader instead of contending for the counter one by one
     const unsigned act = __activemask();
@@ -79,21 +80,22 @@ __device__ __forceinline__ void sort_count_one(const RunDev &rd, int s, int64_t 
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(same) - 1;
     int base = 0;
-    if (lane == leader) base = atomicAdd(rd.sc.cnt + key, __popc(same));
+    if (lane == leader) base = atomicAdd(sc.cnt + key, __popc(same));
     base = __shfl_sync(same, base, leader);
-    rd.sc.slot[p] = base + __popc(same & ((1u << lane) - 1u));
+    sc.slot[p] = base + __popc(same & ((1u << lane) - 1u));
 }
 
 // 2. particles of tile t (block-wide, one thread per cell of the tile)
-__device__ __forceinline__ void sort_tile_sum_block(const RunDev &rd, int64_t t)
+__device__ __forceinline__ void sort_tile_sum_block(const RunDev &rd, const SortScratch &sc,
+                                                    int64_t t)
 {
     const int TC = rd.tile[0] * rd.tile[1] * rd.tile[2];
     __shared__ int tot;
     int v = 0;
-    for (int c = threadIdx.x; c < TC; c += blockDim.x) v += rd.sc.cnt[t * TC + c];
+    for (int c = threadIdx.x; c < TC; c += blockDim.x) v += sc.cnt[t * TC + c];
     (void)sort_block_excl_scan(v, &tot);
     __syncthreads();
-    if (threadIdx.x == 0) rd.sc.tile_count[t] = tot;
+    if (threadIdx.x == 0) sc.tile_count[t] = tot;
 }
 
 // 3. exclusive scan of tile_count[0..nt) into start[0..nt] (block-wide, chunked)
@@ -135,41 +137,61 @@ __device__ __forceinline__ void sort_scan_block(const int64_t *cnt, int64_t *sta
     if (threadIdx.x == 0) start[nt] = carry;
 }
 
-// 4. first position of every cell of tile t and, slot-major, of every (cell, slot)
-//    (block-wide with at least TC threads)
-__device__ __forceinline__ void sort_layout_block(const RunDev &rd, const int64_t *tile_start,
-                                                  int64_t t)
+// 4. first position of every cell of tile t, which starts at position base, and, slot-major, of
+//    every (cell, slot) (block-wide with at least TC threads); returns the tile's particles
+__device__ __forceinline__ int sort_layout_block(const RunDev &rd, const SortScratch &sc,
+                                                 int64_t base, int64_t t)
 {
     const int TC = rd.tile[0] * rd.tile[1] * rd.tile[2];
     const int c = threadIdx.x;
     __shared__ int tot;
     __shared__ int maxc;
-    const int cnt = (c < TC) ? rd.sc.cnt[t * TC + c] : 0;
+    const int cnt = (c < TC) ? sc.cnt[t * TC + c] : 0;
     if (threadIdx.x == 0) maxc = 0;
     __syncthreads();
     if (cnt > 0) atomicMax(&maxc, cnt);
     const int first = sort_block_excl_scan(cnt, &tot);
-    const int64_t base = tile_start[t];
-    if (c < TC) rd.sc.cell_first[t * TC + c] = (int32_t)(base + first);
-    if (!rd.slot_major) return;
+    const int all = tot;
+    if (c < TC) sc.cell_first[t * TC + c] = (int32_t)(base + first);
+    if (!rd.slot_major) return all;
     __syncthreads();
     const int ms = maxc;
     int goff = 0;
     for (int s = 0; s < ms; ++s) {
         const int flag = (cnt > s) ? 1 : 0;
         const int rank = sort_block_excl_scan(flag, &tot);
-        if (flag) rd.sc.pos[base + first + s] = (int32_t)(base + goff + rank);
+        if (flag) sc.pos[base + first + s] = (int32_t)(base + goff + rank);
         goff += tot;
         __syncthreads();
+    }
+    return all;
+}
+
+// 2 to 4 in one stage for a grid of few keys: the block of tile t sums the counts of the tiles
+// before it itself.
+__device__ __forceinline__ void sort_start_layout_block(const RunDev &rd, const SortScratch &sc,
+                                                        int64_t *start, int64_t t)
+{
+    const int before = (int)t * rd.tile[0] * rd.tile[1] * rd.tile[2];
+    __shared__ int sum;
+    int v = 0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < before; i += blockDim.x) v += sc.cnt[i];
+    (void)sort_block_excl_scan(v, &sum);
+    const int base = sum;
+    const int all = sort_layout_block(rd, sc, base, t);
+    if (threadIdx.x == 0) {
+        start[t] = base;
+        if (t + 1 == rd.ntiles) start[rd.ntiles] = base + all;
     }
 }
 
 // 5. the index of particle p at its provisional place in its cell's segment of the cell-major
 //    order (the segment of key k is cell_first[k] .. cell_first[k] + cnt[k] - 1)
-__device__ __forceinline__ void sort_place_one(const RunDev &rd, int64_t p)
+__device__ __forceinline__ void sort_place_one(const SortScratch &sc, int64_t p)
 {
-    const int k = rd.sc.key[p];
-    rd.sc.idx[(int64_t)rd.sc.cell_first[k] + rd.sc.slot[p]] = (int32_t)p;
+    const int k = sc.key[p];
+    sc.idx[(int64_t)sc.cell_first[k] + sc.slot[p]] = (int32_t)p;
 }
 
 // 6. cell-major position r: the particle p placed there by stage 5 is moved to the position of
@@ -178,19 +200,21 @@ __device__ __forceinline__ void sort_place_one(const RunDev &rd, int64_t p)
 //    by (tile, cell, previous index), or in the slot-major order by (tile, rank, cell).  The
 //    threads of a warp usually share a segment, so its loads are broadcasts; the cost grows
 //    with the square of a cell's occupancy.
-__device__ __forceinline__ void sort_scatter_one(const RunDev &rd, int s, int64_t r,
-                                                 void *const *dp, void *const *dm, int32_t *dcell)
+__device__ __forceinline__ void sort_scatter_one(const RunDev &rd, const SortScratch &sc, int s,
+                                                 int64_t r)
 {
     const SpeciesDev &sp = rd.sp[s];
-    const int32_t p = rd.sc.idx[r];
-    const int k = rd.sc.key[p];
-    const int64_t first = rd.sc.cell_first[k];
-    const int m = rd.sc.cnt[k];
-    const int32_t *seg = rd.sc.idx + first;
+    void *const *dp = sp.pos_alt, *const *dm = sp.mom_alt;
+    int32_t *dcell = sp.cell_alt;
+    const int32_t p = sc.idx[r];
+    const int k = sc.key[p];
+    const int64_t first = sc.cell_first[k];
+    const int m = sc.cnt[k];
+    const int32_t *seg = sc.idx + first;
     int rank = 0;
     for (int j = 0; j < m; ++j) rank += (__ldg(seg + j) < p) ? 1 : 0;
     const int64_t rr = first + rank;
-    const int64_t q = rd.slot_major ? (int64_t)rd.sc.pos[rr] : rr;
+    const int64_t q = rd.slot_major ? (int64_t)sc.pos[rr] : rr;
     if (rd.prec == 1) {
         dcell[q] = sp.cell[p];
         for (int a = 0; a < rd.dim; ++a) ((float *)dp[a])[q] = ((const float *)sp.pos[a])[p];
