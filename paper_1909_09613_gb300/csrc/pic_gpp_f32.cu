@@ -10,7 +10,10 @@ template <int L, int KT, bool DET>
 __global__ void __launch_bounds__(256, 2) k_gpp2d(const __grid_constant__ RunDev rd)
 {
     extern __shared__ __align__(16) char smem[];
-    tile_2d<L, KT, float, DET>(rd, smem, blockIdx.x);
+    for (int64_t t = blockIdx.x * rd.ntiles / gridDim.x; t * gridDim.x < (blockIdx.x + 1) * rd.ntiles; ++t) {
+        tile_2d<L, KT, float, DET>(rd, smem, t, nullptr, EvenSplit{t, rd.ntiles});
+        __syncthreads();  // the next tile is staged over this one
+    }
 }
 
 template <int L, int KT>
@@ -20,7 +23,7 @@ cudaError_t go(const RunDev &rd, cudaStream_t st)
     auto k = rd.det ? k_gpp2d<L, KT, true> : k_gpp2d<L, KT, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3((unsigned)rd.ntiles, tile_parts(rd)), 256, smem, st>>>(rd);
+    k<<<tile_ctas(rd), 256, smem, st>>>(rd);
     return cudaGetLastError();
 }
 

@@ -763,38 +763,50 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     ((float *)hs.pos1)[p] = o[1];
 }
 
-// Which share of a tile's particles a CTA takes: part() of parts(), read where used so that it
-// holds no registers across the tile.  A single run's launch puts the part in blockIdx.y
-// (tile_parts chooses how many); the batched kernel keeps it in shared memory beside its work
-// item.
+// Which share of a tile's particles a CTA takes: [from, to) of `of` equal shares of every species'
+// range, read where used so that it holds no registers across the tile.  The FP64 form's launch
+// puts the part in blockIdx.y (tile_parts chooses how many); the FP32 form's divides the grid's
+// tiles evenly over its CTAs, tile borders or not (tile_ctas); the batched kernel keeps the part in
+// shared memory beside its work item.
 struct GridSplit {
-    __device__ __forceinline__ int part() const { return (int)blockIdx.y; }
-    __device__ __forceinline__ int parts() const { return (int)gridDim.y; }
+    __device__ __forceinline__ int64_t from() const { return blockIdx.y; }
+    __device__ __forceinline__ int64_t to() const { return blockIdx.y + 1; }
+    __device__ __forceinline__ int64_t of() const { return gridDim.y; }
+};
+struct EvenSplit {
+    int64_t tile, ntiles;  // CTA k of G takes k ntiles / G .. (k + 1) ntiles / G
+    __device__ __forceinline__ int64_t from() const
+    {
+        return max(blockIdx.x * ntiles - tile * gridDim.x, (int64_t)0);
+    }
+    __device__ __forceinline__ int64_t to() const
+    {
+        return min((blockIdx.x + 1) * ntiles - tile * gridDim.x, (int64_t)gridDim.x);
+    }
+    __device__ __forceinline__ int64_t of() const { return gridDim.x; }
 };
 struct SharedSplit {
     const int *s;  // (part, parts)
-    __device__ __forceinline__ int part() const { return s[0]; }
-    __device__ __forceinline__ int parts() const { return s[1]; }
+    __device__ __forceinline__ int64_t from() const { return s[0]; }
+    __device__ __forceinline__ int64_t to() const { return s[0] + 1; }
+    __device__ __forceinline__ int64_t of() const { return s[1]; }
 };
 
 template <typename Split>
 __device__ __forceinline__ void split_range(const Split &split, int64_t &a, int64_t &b)
 {
-    if (split.parts() > 1) {
-        const int64_t len = b - a;
-        const int part = split.part(), parts = split.parts();
-        b = a + (len * (part + 1)) / parts;
-        a += (len * part) / parts;
-    }
+    const int64_t len = b - a, of = split.of();
+    if (split.to() - split.from() == of) return;
+    b = a + len * split.to() / of;
+    a += len * split.from() / of;
 }
 
-// All particles of one tile (both species), 2D FP32 form.  tt_shared as in stage2d_carve.  With
-// split.parts() > 1 only that part of every species' particles of the tile (a contiguous share
-// of its range): a grid of few tiles, or a batch of few particles, is spread over several CTAs
-// per tile, each staging the tile and adding its own share of the current.
-template <int L, int KT, typename R, bool DET = false, typename Split = GridSplit>
-__device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile,
-                        const TTable *tt_shared = nullptr, const Split split = Split())
+// All particles of one tile (both species), 2D FP32 form, or split's share of them: a grid of few
+// tiles, or a batch of few particles, is spread over several CTAs per tile, each staging the tile
+// and adding its own share of the current.  tt_shared as in stage2d_carve.
+template <int L, int KT, typename R, bool DET = false, typename Split>
+__device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile, const TTable *tt_shared,
+                        const Split split)
 {
     Stage2D<R> st = stage2d_carve<R>(smem, rd.reg_nodes, tt_shared, DET);
     const int tx = (int)(tile % rd.ntile[0]);

@@ -7,34 +7,65 @@ namespace pic {
 bool build_ttable(int l, int scheme, double dtt, TTable *t, bool fixed = false);
 int ttable_eval_host(const TTable *t, int l, double delta, double *w);
 
-// CTAs per tile of a single run's 2D particle pass (tile_2d's split), from the tile and particle
-// counts.  A grid of few tiles left most SMs idle: 64x32 cells are 4 to 8 tiles, 256x128 are 64,
-// on 304 CTA slots (two per SM).  Every tile takes as many parts as fill the slots once, down to
-// one warp of each species per part (particle kernel, us, one CTA per tile -> this rule: FP64
-// 64x32 quadratic at 4 per cell 105 -> 21, FP32 50 -> 23, FP32 250x126 cubic at 8 per cell 85 ->
-// 44, FP32 256x128 quartic at 64 per cell 445 -> 173).  The FP64 form, bound by a pipe every CTA
-// of the SM shares, also splits a grid of few waves so that its last wave is short, while a part
-// keeps 256 particles of a species (512x256 cubic at 64 per cell: 7388 -> 6362 us); the FP32 form
-// loses there to the parts' extra stages and flushes (256 tiles: 421 us with one part, 432 with
-// two) and stays at one wave.
-inline unsigned tile_parts(const RunDev &rd)
+// CTA slots of the 2D particle passes (two per SM); 0 if the device does not say.
+inline int64_t tile_slots()
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess
         || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
+        return 0;
+    return 2 * (int64_t)sms;
+}
+
+// particles of the fullest species per tile
+inline int64_t tile_load(const RunDev &rd)
+{
     int64_t n = 0;
     for (int s = 0; s < rd.nsp; ++s) n = rd.sp[s].n > n ? rd.sp[s].n : n;
-    const int64_t slots = 2 * (int64_t)sms, per_tile = (n + rd.ntiles - 1) / rd.ntiles;
+    return (n + rd.ntiles - 1) / rd.ntiles;
+}
+
+// CTAs per tile of a single FP64 run's 2D particle pass (tile_fx's split).  A grid of few tiles
+// left most SMs idle: 64x32 cells are 8 tiles on 304 CTA slots.  Every tile takes as many parts
+// as fill the slots once, down to one warp of each species per part (64x32 quadratic at 4 per
+// cell 105 -> 21 us).  Bound by a pipe every CTA of the SM shares, this form also splits a grid of
+// few waves so that its last wave is short, while a part keeps 256 particles of a species
+// (512x256 cubic at 64 per cell: 7388 -> 6362 us).
+inline unsigned tile_parts(const RunDev &rd)
+{
+    const int64_t slots = tile_slots(), per_tile = tile_load(rd);
     int64_t parts = slots / rd.ntiles;
-    if (rd.prec == 0) {
-        const int64_t want = (8 * slots + rd.ntiles - 1) / rd.ntiles, most = per_tile / 256;
-        const int64_t p = want < most ? want : most;
-        if (p > parts) parts = p;
-    }
+    const int64_t want = (8 * slots + rd.ntiles - 1) / rd.ntiles, full = per_tile / 256;
+    const int64_t p = want < full ? want : full;
+    if (p > parts) parts = p;
     const int64_t most = (per_tile + 31) / 32;
     if (parts > most) parts = most;
     return (unsigned)(parts > 1 ? parts : 1);
+}
+
+// particles of the fullest species a CTA keeps when the tiles are divided evenly (tile_ctas)
+constexpr int64_t kEvenMin = 1024;
+
+// CTAs of a single FP32 run's 2D particle pass; every CTA takes the same share of the grid's tiles
+// (EvenSplit).  Whole tiles or whole parts of them left slots empty in a grid of few waves: 256
+// tiles, or 64 tiles in 4 parts, are 256 CTAs on 304 slots.  A share that crosses a tile border
+// stages twice and still wins (particle kernel, us, 512x256 at 32 per cell: quadratic 212 -> 193,
+// cubic 229 -> 200; 256x128 quartic at 64 per cell 168 -> 162).
+inline unsigned tile_ctas(const RunDev &rd)
+{
+    const int64_t slots = tile_slots(), per_tile = tile_load(rd), nt = rd.ntiles;
+    // whole parts per tile, as many as fill the slots once, down to one warp of each species
+    int64_t parts = slots / nt;
+    const int64_t most = (per_tile + 31) / 32;
+    if (parts > most) parts = most;
+    if (parts < 1) parts = 1;
+    // all slots of the last wave, where that leaves a CTA enough particles to pay for staging a
+    // second tile and the waves are few
+    if (slots > 0) {
+        const int64_t waves = (nt * parts + slots - 1) / slots, g = slots * waves;
+        if (waves <= 4 && 16 * g >= 17 * nt * parts && per_tile * nt / g >= kEvenMin) return (unsigned)g;
+    }
+    return (unsigned)(nt * parts);
 }
 // fused gather-push-deposit over all tiles of one run
 cudaError_t launch_gpp(const RunDev &rd, int kt, cudaStream_t st);
