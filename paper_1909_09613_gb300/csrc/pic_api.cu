@@ -244,6 +244,14 @@ void set_det_scale(pic_ctx *c)
     rd.det_inv64 = std::ldexp(1.0, 31) / sc;
 }
 
+// Kernels of a charge density (none without particles).
+int rho_launches(const RunDev &rd)
+{
+    for (int s = 0; s < rd.nsp; ++s)
+        if (rd.sp[s].n > 0) return 1;
+    return 0;
+}
+
 // Record G = D.E - rho of the current state as the reference of the Gauss-residual drift.
 int capture_gauss_ref(pic_ctx *c)
 {
@@ -251,8 +259,7 @@ int capture_gauss_ref(pic_ctx *c)
     refresh_species_ptrs(c);
     if (launch_gauss_ref(c->rd, c->rho, c->gref, c->diag_out, c->stream) != cudaSuccess)
         return PIC_ECUDA;
-    c->kernel_launches += 2;
-    for (int s = 0; s < c->rd.nsp; ++s) c->kernel_launches += c->rd.sp[s].n > 0 ? 1 : 0;
+    c->kernel_launches += 1 + rho_launches(c->rd);
     c->gref_valid = true;
     return PIC_OK;
 }
@@ -952,7 +959,7 @@ int pic_diag(pic_ctx *c, pic_diag_t *out)
     if (launch_diag(rd, c->diag_out, c->rho, c->gref_valid ? c->gref : nullptr,
                     cont ? c->rho_prev : nullptr, c->stream) != cudaSuccess)
         return PIC_ECUDA;
-    c->kernel_launches += 2 + 2 * rd.nsp;
+    c->kernel_launches += 2 + rd.nsp + rho_launches(rd);
     // this rho is the reference of the next call's continuity residual
     if (cudaMemcpyAsync(c->rho_prev, c->rho, rd.ncell * sizeof(double), cudaMemcpyDeviceToDevice,
                         c->stream) != cudaSuccess)

@@ -382,6 +382,17 @@ __device__ __forceinline__ int wrap_near(int i, int n)
     return (i < 0 || i >= n) ? wrap_idx(i, n) : i;
 }
 
+// Local coordinate of a cell index along one axis, relative to the tile origin, taking the
+// periodic image that lies within [-D, tile + D).  Returns false if none does.
+__device__ __forceinline__ bool local_coord(int c, int origin, int tile, int drift, int n, int &lc)
+{
+    int l = c - origin;
+    if (l < -drift) l += n;
+    if (l >= tile + drift) l -= n;
+    lc = l;
+    return l >= -drift && l < tile + drift;
+}
+
 __device__ __forceinline__ void set_err(int32_t *err, int bit)
 {
     if (err) atomicOr(err, bit);

@@ -200,17 +200,6 @@ __device__ void stage2d_flush(const RunDev &rd, const Stage2D<R> &st, int x0, in
     }
 }
 
-// Local coordinate of a cell index along one axis, relative to the tile origin, taking the
-// periodic image that lies within [-D, tile + D).  Returns false if none does.
-__device__ __forceinline__ bool local_coord(int c, int origin, int tile, int drift, int n, int &lc)
-{
-    int l = c - origin;
-    if (l < -drift) l += n;
-    if (l >= tile + drift) l -= n;
-    lc = l;
-    return l >= -drift && l < tile + drift;
-}
-
 // Add (a, b) to the two FP32 values at p (8-byte aligned: two neighbouring x nodes of a staged
 // row that starts at an even node) with one 64-bit compare-and-swap loop and a packed add, each
 // half rounded as the scalar add.  Shared-memory FP32 additions are compare-and-swap loops
