@@ -28,7 +28,7 @@ struct TTable {
     double phib;      // interior breakpoint (0 if none)
     union {
         double coef[2][PIC_TK_MAX][5];
-        // 2D FP64 form: the coefficients of the polynomial in s = t / h, h the length of the
+        // FP64 form: the coefficients of the polynomial in s = t / h, h the length of the
         // sub-interval, in units of 2^-59 (pic_fixed.cuh)
         int64_t ci[2][PIC_TK_MAX][5];
     };
@@ -37,7 +37,7 @@ struct TTable {
         // FP32 form: coef in FP32, grouped for vector loads: cf4[p][m][g] = coefficient m of
         // nodes 4g .. 4g + 3
         float4 cf4[2][5][2];
-        // 2D FP64 form: Rfrac and phib in units of 2^-64, and 1 / h = 2^shift (1 + invm1) per
+        // FP64 form: Rfrac and phib in units of 2^-64, and 1 / h = 2^shift (1 + invm1) per
         // sub-interval (invm1 in units of 2^-62)
         struct {
             uint64_t rfrac, phib, invm1[2];
@@ -199,19 +199,18 @@ __device__ __forceinline__ void det_words64(double v, double inv, unsigned long 
 // psi in [0,1); node k (k = 0..L) sits at distance (L-1)/2 + psi - k from the particle.
 // These are the uniform B-spline basis polynomials written in the local variable psi.
 // ------------------------------------------------------------------------------------------
-template <int L, typename R>
-__device__ __forceinline__ void bspline(R p, R *w)
+template <int L>
+__device__ __forceinline__ void bspline(float p, float *w)
 {
-    const R one = R(1);
-    const R q = one - p;
+    const float q = 1.0f - p;
     if constexpr (L == 1) {
         w[0] = q;
         w[1] = p;
     } else if constexpr (L == 2) {
-        w[0] = R(0.5) * q * q;
-        w[1] = R(0.5) + p * q;
-        w[2] = R(0.5) * p * p;
-    } else if constexpr (L == 3 && sizeof(R) == 4) {
+        w[0] = 0.5f * q * q;
+        w[1] = 0.5f + p * q;
+        w[2] = 0.5f * p * p;
+    } else if constexpr (L == 3) {
         // node k at psi is node L - k at 1 - psi: (w3, w0) and (w1, w2) are one polynomial
         // each, evaluated on the pair (psi, 1 - psi) with packed FP32 arithmetic
         const float2 pq = make_float2(p, q);
@@ -223,16 +222,7 @@ __device__ __forceinline__ void bspline(R p, R *w)
         w[1] = m.x;
         w[2] = m.y;
         w[3] = e.x;
-    } else if constexpr (L == 3) {
-        // Horner forms of w3 = psi^3/6 and w1 = 2/3 - psi^2 (1 - psi/2); w0 and w2 are the same
-        // polynomials in 1 - psi (node k at psi is node 3 - k at 1 - psi): eleven FP64 operations
-        const R p2 = p * p;
-        const R q2 = q * q;
-        w[0] = q2 * (q * R(1.0 / 6.0));
-        w[1] = (R(0.5) * p - one) * p2 + R(2.0 / 3.0);
-        w[2] = (R(0.5) * q - one) * q2 + R(2.0 / 3.0);
-        w[3] = p2 * (p * R(1.0 / 6.0));
-    } else if constexpr (sizeof(R) == 4) {
+    } else {
         // L = 4 on the pair (psi, 1 - psi): (w4, w0) = (psi^4, (1-psi)^4) / 24, and (w3, w1) one
         // Horner polynomial; the middle weight from the partition of unity (>= 11/24)
         const float2 pq = make_float2(p, q);
@@ -248,66 +238,22 @@ __device__ __forceinline__ void bspline(R p, R *w)
         w[3] = t.x;
         w[4] = e.x;
         w[2] = 1.0f - (((w[0] + w[1]) + w[3]) + w[4]);
-    } else {
-        // Horner forms with the 1/24 folded into the coefficients; the middle weight from the
-        // partition of unity (it is >= 11/24)
-        const R p2 = p * p;
-        const R q2 = q * q;
-        w[0] = q2 * (q2 * R(1.0 / 24.0));
-        w[1] = (((R(-1.0 / 6.0) * p + R(0.5)) * p - R(0.25)) * p - R(0.5)) * p + R(11.0 / 24.0);
-        w[3] = (((R(-1.0 / 6.0) * p + R(1.0 / 6.0)) * p + R(0.25)) * p + R(1.0 / 6.0)) * p
-               + R(1.0 / 24.0);
-        w[4] = p2 * (p2 * R(1.0 / 24.0));
-        w[2] = one - (((w[0] + w[1]) + w[3]) + w[4]);
     }
-}
-
-// Comparisons of non-negative FP64 values against non-negative constants, taken on the bit
-// pattern: for x >= +0 and c >= +0, x >= c exactly when bits(x) >= bits(c) as integers, and for
-// c = 1/2 or 1 (low word zero) the high words decide.  The FP64 pipe of this GPU completes two
-// lanes per clock per SM, so an integer compare here frees one of its issue slots; R = float
-// keeps the plain compare.  (A NaN offset only selects a branch whose indices stay in range.)
-template <typename R>
-__device__ __forceinline__ bool ge_half(R x)
-{
-    if constexpr (sizeof(R) == 8) return __double2hiint(x) >= 0x3FE00000;
-    else return x >= R(0.5);
-}
-
-template <typename R>
-__device__ __forceinline__ bool ge_one(R x)
-{
-    if constexpr (sizeof(R) == 8) return __double2hiint(x) >= 0x3FF00000;
-    else return x >= R(1);
-}
-
-template <typename R>
-__device__ __forceinline__ bool ge_pos(R x, R c)
-{
-    if constexpr (sizeof(R) == 8) return __double_as_longlong(x) >= __double_as_longlong(c);
-    else return x >= c;
-}
-
-template <typename R>
-__device__ __forceinline__ bool is_neg(R x)  // x < 0 for x != -0 (the callers never see -0)
-{
-    if constexpr (sizeof(R) == 8) return __double2hiint(x) < 0;
-    else return x < R(0);
 }
 
 // Split an offset delta in [0,1) against a node lattice shifted by h = c + (L-1)/2 (c = 0 for
 // integer nodes, 1/2 for half-integer nodes): returns the first node (relative to the cell)
 // and the local coordinate psi in [0,1).
-template <int L, typename R>
-__device__ __forceinline__ int spline_base(R delta, bool half, R &psi)
+template <int L>
+__device__ __forceinline__ int spline_base(float delta, bool half, float &psi)
 {
     // h2 = 2h is an integer: 2c + L - 1
     const int h2 = (half ? 1 : 0) + L - 1;
     const int hi = h2 >> 1;            // integer part of h
     if (h2 & 1) {                      // h = hi + 1/2
-        if (ge_half(delta)) { psi = delta - R(0.5); return -hi; }
-        psi = delta + R(0.5);
-        if (ge_one(psi)) { psi = R(0); return -hi; }  // delta + 1/2 rounded up to 1
+        if (delta >= 0.5f) { psi = delta - 0.5f; return -hi; }
+        psi = delta + 0.5f;
+        if (psi >= 1.0f) { psi = 0.0f; return -hi; }  // delta + 1/2 rounded up to 1
         return -hi - 1;
     }
     psi = delta;
@@ -316,53 +262,37 @@ __device__ __forceinline__ int spline_base(R delta, bool half, R &psi)
 
 // Weights of the integer-node factor from a TTable (WT: T_l, MC: W_l).  Returns the first
 // node relative to the cell; w[0..KT-1] (entries beyond the table's K are zero).
-template <int L, int KT, typename R>
-__device__ __forceinline__ int ttable_weights(const TTable &t, R delta, R *w)
+template <int L, int KT>
+__device__ __forceinline__ int ttable_weights(const TTable &t, float delta, float *w)
 {
-    R v;
-    if constexpr (sizeof(R) == 8) v = delta - R(t.Rfrac);
-    else v = delta - R(t.Rfrac_f);
-    // v in (-1, 1)
+    const float v = delta - t.Rfrac_f;  // in (-1, 1)
     int fl = 0;
-    R phi = v;
-    if (is_neg(v)) {  // v = delta - Rfrac is never -0 (delta = Rfrac gives +0)
-        phi = v + R(1);
+    float phi = v;
+    if (v < 0.0f) {
+        phi = v + 1.0f;
         fl = -1;
-        if (ge_one(phi)) { phi = R(0); fl = 0; }
+        if (phi >= 1.0f) { phi = 0.0f; fl = 0; }
     }
     const int base = fl - t.Rint + 1;
-    R phib;
-    if constexpr (sizeof(R) == 8) phib = R(t.phib);
-    else phib = R(t.phib_f);
-    const int p = ge_pos(phi, phib) ? 1 : 0;  // phi >= +0, phib >= +0
-    const R tl = phi - (p ? phib : R(0));
-    if constexpr (sizeof(R) == 8) {
+    const int p = phi >= t.phib_f ? 1 : 0;
+    const float tl = phi - (p ? t.phib_f : 0.0f);
+    // the Horner steps for four nodes at a time: one 16-byte shared load per coefficient and two
+    // packed FMAs (each rounded as the scalar FMA)
+    const float2 t2 = make_float2(tl, tl);
 #pragma unroll
-        for (int k = 0; k < KT; ++k) {
-            R acc = R(t.coef[p][k][L]);
+    for (int g = 0; g < (KT + 3) / 4; ++g) {
+        float4 c = t.cf4[p][L][g];
+        float2 a01 = make_float2(c.x, c.y), a23 = make_float2(c.z, c.w);
 #pragma unroll
-            for (int m = L - 1; m >= 0; --m) acc = acc * tl + R(t.coef[p][k][m]);
-            w[k] = acc;
+        for (int m = L - 1; m >= 0; --m) {
+            c = t.cf4[p][m][g];
+            a01 = __ffma2_rn(a01, t2, make_float2(c.x, c.y));
+            a23 = __ffma2_rn(a23, t2, make_float2(c.z, c.w));
         }
-    } else {
-        // the same Horner steps for four nodes at a time: one 16-byte shared load per
-        // coefficient and two packed FMAs (each rounded as the scalar FMA)
-        const float2 t2 = make_float2(tl, tl);
+        const float u[4] = {a01.x, a01.y, a23.x, a23.y};
 #pragma unroll
-        for (int g = 0; g < (KT + 3) / 4; ++g) {
-            float4 c = t.cf4[p][L][g];
-            float2 a01 = make_float2(c.x, c.y), a23 = make_float2(c.z, c.w);
-#pragma unroll
-            for (int m = L - 1; m >= 0; --m) {
-                c = t.cf4[p][m][g];
-                a01 = __ffma2_rn(a01, t2, make_float2(c.x, c.y));
-                a23 = __ffma2_rn(a23, t2, make_float2(c.z, c.w));
-            }
-            const float v[4] = {a01.x, a01.y, a23.x, a23.y};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (4 * g + j < KT) w[4 * g + j] = v[j];
-        }
+        for (int j = 0; j < 4; ++j)
+            if (4 * g + j < KT) w[4 * g + j] = u[j];
     }
     return base;
 }

@@ -29,41 +29,6 @@ struct PState {
     R u[3];
 };
 
-// ---- particle storage ---------------------------------------------------------------------
-
-template <int DIM, typename R>
-__device__ __forceinline__ void load_particle(const RunDev &rd, const SpeciesDev &sp, int64_t p,
-                                              PState<R> &s)
-{
-    if constexpr (sizeof(R) == 4) {
-        const int c = __ldg(sp.cell + p);
-        if constexpr (DIM == 2) {
-            s.c[1] = fast_div(c, rd.div_n0.m, rd.div_n0.s);
-            s.c[0] = c - s.c[1] * rd.n[0];
-            s.c[2] = 0;
-        } else {
-            const int nxy = rd.n[0] * rd.n[1];
-            s.c[2] = fast_div(c, rd.div_n01.m, rd.div_n01.s);
-            const int r = c - s.c[2] * nxy;
-            s.c[1] = fast_div(r, rd.div_n0.m, rd.div_n0.s);
-            s.c[0] = r - s.c[1] * rd.n[0];
-        }
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) s.d[a] = __ldg((const float *)sp.pos[a] + p);
-    } else {
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            const double x = __ldg((const double *)sp.pos[a] + p);
-            const double f = floor(x);
-            s.c[a] = min(max((int)f, 0), rd.n[a] - 1);  // a non-finite position stays in range
-            s.d[a] = x - f;
-        }
-        if (DIM == 2) s.c[2] = 0;
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) s.u[a] = __ldg((const R *)sp.mom[a] + p);
-}
-
 // ---- weights of one axis: W_l at half-integer nodes (Eq. shape-real), T_l of Eq. tau_l (WT) or
 // W_l (MC) at integer nodes -------------------------------------------------------------------
 
@@ -79,9 +44,9 @@ template <int L, int KT, typename R>
 __device__ __forceinline__ void axis_weights(const TTable &tt, R d, AxisW<L, KT, R> &w)
 {
     R psi;
-    w.bh = spline_base<L, R>(d, true, psi);
-    bspline<L, R>(psi, w.wh);
-    w.bt = ttable_weights<L, KT, R>(tt, d, w.wt);
+    w.bh = spline_base<L>(d, true, psi);
+    bspline<L>(psi, w.wh);
+    w.bt = ttable_weights<L, KT>(tt, d, w.wt);
 }
 
 // Esirkepov window of one axis: S0 (old-position weights) and DS = S1 - S0 on l+2 nodes
@@ -93,29 +58,6 @@ struct AxisS {
     R s0[L + 2];
     R ds[L + 2];
 };
-
-// FP64: S1 from the stored new position (cell shift sh, offset o_new), DS = S1 - S0.
-template <int L, typename R>
-__device__ __forceinline__ void axis_shapes(R d_old, int sh, R o_new, AxisS<L, R> &s)
-{
-    R p0, p1, w0[L + 1], w1[L + 1];
-    const int b0 = spline_base<L, R>(d_old, false, p0);
-    const int b1 = sh + spline_base<L, R>(o_new, false, p1);
-    bspline<L, R>(p0, w0);
-    bspline<L, R>(p1, w1);
-    s.wb = min(b0, b1);
-    s.wide = b0 != b1;
-    const bool sh0 = b0 > s.wb, sh1 = b1 > s.wb;
-#pragma unroll
-    for (int k = 0; k < L + 2; ++k) {
-        const R a0 = (k <= L) ? w0[k] : R(0);
-        const R a1 = (k >= 1) ? w0[k - 1] : R(0);
-        const R c0 = (k <= L) ? w1[k] : R(0);
-        const R c1 = (k >= 1) ? w1[k - 1] : R(0);
-        s.s0[k] = sh0 ? a1 : a0;
-        s.ds[k] = (sh1 ? c1 : c0) - s.s0[k];
-    }
-}
 
 // Divided difference (P_k(b) - P_k(a)) / (b - a) of the B-spline basis polynomials of
 // bspline<L> (monomial coefficients in psi), evaluated without cancellation for a, b in [0,1].
@@ -167,8 +109,8 @@ template <int L, bool COLLECTIVE = false>
 __device__ __forceinline__ void axis_shapes_dd(float d_old, float delta, AxisS<L, float> &s)
 {
     float p0, w0[L + 1];
-    const int b0 = spline_base<L, float>(d_old, false, p0);
-    bspline<L, float>(p0, w0);
+    const int b0 = spline_base<L>(d_old, false, p0);
+    bspline<L>(p0, w0);
     const float p1 = p0 + delta;
     const bool up = p1 >= 1.0f, dn = p1 < 0.0f;
     if (COLLECTIVE ? !__any_sync(0xffffffffu, up || dn) : !(up || dn)) {
@@ -236,52 +178,18 @@ __device__ __forceinline__ R boris(R h, const R *E, const R *B, R *u)
     return rsqrt_r(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
 }
 
-// Move one axis in cell units, x^{n+1} = x^n + dt u^{n+1/2} / gamma^{n+1/2} (App. E): returns
-// the cell shift sh in {-1,0,1} and the new offset o in [0,1).  In the FP64 form o is re-derived
-// from the stored value cell + o so that the next step's old-position weights are bit-identical
-// to this step's new-position weights; xs is that stored value (unused for FP32).
-template <typename R>
-__device__ __forceinline__ int move_axis(R d, R delta, int c, int n, R &o, int &cn, R &xs)
+// Move one axis in cell units, x^{n+1} = x^n + dt u^{n+1/2} / gamma^{n+1/2} (App. E): the new offset
+// o in [0,1) and cell cn.
+__device__ __forceinline__ void move_axis(float d, float delta, int c, int n, float &o, int &cn)
 {
-    const R xn = d + delta;
-    int sh;
-    R on;
-    if constexpr (sizeof(R) == 8) {
-        // xn - sh as xn plus a selected constant: the same rounding, without converting sh.
-        // The compares are taken on the bit pattern (is_neg, ge_one): for finite values they
-        // decide as the FP64 compares do (-0 aside, which moves to +0 here); a NaN position,
-        // which only a non-finite momentum makes, leaves with a finite offset and a cell shift
-        // of at most 1, while its current and kinetic energy carry the NaN that reports it.
-        const bool lo = is_neg(xn), up = ge_one(xn);
-        sh = lo ? -1 : (up ? 1 : 0);
-        on = xn + (lo ? 1.0 : (up ? -1.0 : 0.0));
-        if (ge_one(on)) { on = 0.0; sh = min(sh + 1, 1); }  // finite: only from sh = -1
-        if (is_neg(on)) on = 0.0;
-    } else {
-        sh = (xn < R(0)) ? -1 : ((xn >= R(1)) ? 1 : 0);
-        on = xn - R(sh);
-        if (on >= R(1)) { on = R(0); sh += 1; }
-        if (on < R(0)) on = R(0);
-    }
-    int cc = c + sh;
-    if (cc < 0) cc += n;
-    if (cc >= n) cc -= n;
-    xs = R(0);
-    if constexpr (sizeof(R) == 8) {
-        const double stored = (double)cc + on;
-        double o2 = stored - (double)cc;  // exact (Sterbenz)
-        xs = stored;
-        if (ge_one(o2)) {  // cc + on rounded up to the next integer, which is the stored value
-            o2 = 0.0;
-            sh += 1;
-            cc += 1;
-            if (cc >= n) { cc -= n; xs = 0.0; }
-        }
-        on = o2;
-    }
-    o = on;
-    cn = cc;
-    return sh;
+    const float xn = d + delta;
+    int sh = (xn < 0.0f) ? -1 : ((xn >= 1.0f) ? 1 : 0);
+    o = xn - (float)sh;
+    if (o >= 1.0f) { o = 0.0f; sh += 1; }
+    if (o < 0.0f) o = 0.0f;
+    cn = c + sh;
+    if (cn < 0) cn += n;
+    if (cn >= n) cn -= n;
 }
 
 }  // namespace pic

@@ -144,12 +144,12 @@ __device__ __forceinline__ void particle_3d(const RunDev &rd, const SpeciesDev &
 
     // ---- Boris push and move ----
     const R ig = boris<R>(R(sp.qmdt_half), E, B, s.u);
-    R o[3], dl[3], xs;
+    R o[3], dl[3];
     int cn[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         dl[a] = R(rd.dtt[a]) * s.u[a] * ig;
-        move_axis<R>(s.d[a], dl[a], s.c[a], rd.n[a], o[a], cn[a], xs);
+        move_axis(s.d[a], dl[a], s.c[a], rd.n[a], o[a], cn[a]);
     }
 
     // ---- Esirkepov deposit ----

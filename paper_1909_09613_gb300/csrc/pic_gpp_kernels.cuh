@@ -5,10 +5,6 @@
 
 namespace pic {
 
-// Accumulation type of the shared-memory current tile: FP32 in the precision form, FP64 in
-// the plain form.
-template <typename R> struct AccT { typedef R T; };
-
 // Shared-memory layout of a staged 2D tile (all arrays reg_nodes long, x fastest):
 //   pa = (E1, B2) pairs  [both sit at (i+1/2, j): W along x, T along y]
 //   pb = (E2, B1) pairs  [both sit at (i, j+1/2): T along x, W along y]
@@ -658,12 +654,12 @@ __device__ __forceinline__ void particle_2d(const Hot2D h, const HotSp<R> hs,
     const R ig = boris<R>(R(hs.qmdt_half), E, B, s.u);
 
     // ---- move ----
-    R o[2], dl[2], xs[2];
-    int cn[2], shv[2];
+    R o[2], dl[2];
+    int cn[2];
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
         dl[a] = R(a == 0 ? h.dtt0 : h.dtt1) * s.u[a] * ig;
-        shv[a] = move_axis<R>(s.d[a], dl[a], s.c[a], a == 0 ? h.n0 : h.n1, o[a], cn[a], xs[a]);
+        move_axis(s.d[a], dl[a], s.c[a], a == 0 ? h.n0 : h.n1, o[a], cn[a]);
     }
 
     // ---- Esirkepov deposit ----
