@@ -2,10 +2,13 @@
 //
 // One step of the whole batch is a fixed sequence of launches, captured once in a CUDA graph
 // and replayed: a plan kernel decides on the device which runs are due for a tile sort; the
-// batched sort kernels sort only those runs; the current of every run is cleared; ONE
-// persistent gather-push-deposit kernel (one CTA per SM slot) pulls (run, tile) work items,
-// heaviest first, from a device counter and processes them with the same tile code as a single
-// run; three batched Yee launches finish the step.
+// batched sort kernels sort only those runs; ONE persistent gather-push-deposit kernel (one CTA
+// per SM slot) pulls (run, tile) work items, heaviest first, from a device counter and processes
+// them with the same tile code as a single run; two batched Yee launches finish the step.  As in a
+// single run, the half step of B that ends a step and the one that begins the next of the same call
+// are one pass, which also clears the current: two graphs, of a step that another follows and of a
+// call's last step, and one launch ahead of a call's first step (48 uneven runs: two half-step
+// passes of 90 us and a clearing pass of 11 us per step -> one half-step pass).
 //
 // Every launch has a fixed grid and walks device-resident tables (run descriptors, per-stage
 // block maps, work items) whose lengths it reads from device memory.  The captured graph
@@ -223,25 +226,7 @@ __global__ void k_b_swap(const Counts *cn, RunDev *runs, const int *due, int s)
     }
 }
 
-// ---- current cleared, Yee updates ----
-__global__ void __launch_bounds__(kBlock) k_b_zero_j(const Counts *cn, const RunDev *runs,
-                                                     const BlockMap *bm)
-{
-    for (int b = blockIdx.x; b < cn->cell; b += gridDim.x) {
-        const BlockMap m = bm[b];
-        const RunDev &rd = runs[m.run];
-        double *j0 = rd.F[6], *j1 = rd.F[7], *j2 = rd.F[8];
-        for (int k = 0; k < kCellPer; ++k) {
-            const int64_t c = ((int64_t)m.block * kCellPer + k) * blockDim.x + threadIdx.x;
-            if (c < rd.ncell) {
-                j0[c] = 0.0;
-                j1[c] = 0.0;
-                j2[c] = 0.0;
-            }
-        }
-    }
-}
-
+// ---- Yee updates ----
 __global__ void __launch_bounds__(kBlock) k_b_yee_b(const Counts *cn, const RunDev *runs,
                                                     const BlockMap *bm, int flags)
 {
@@ -346,10 +331,10 @@ struct pic_batch {
     BlockMap *d_bm_cell;
     int4 *d_items;
     int *d_counter;
-    // launch shapes and the graph of one step
+    // launch shapes and the graphs of one step: one that another step follows, and a last one
     int grid_runs, grid_scan, grid_stage, grid_tile, grid_gpp;
-    cudaGraphExec_t exec;
-    bool have_graph;
+    cudaGraphExec_t exec[2];
+    bool have_graph[2];
     cudaEvent_t ev0, ev1;
     bool timing;
     int64_t steps_since_sync;
@@ -428,9 +413,18 @@ bool tables_fit(const pic_batch *b, const Tables &t, int n)
              || (int64_t)t.items.size() > b->cap_tile || t.smem > b->smem);
 }
 
-// Launch sequence of one batch step on b->stream (also used while capturing).  Every grid is
-// fixed by the capacities; the kernels read the table lengths from d_counts.
-cudaError_t enqueue_step(pic_batch *b)
+// Ahead of a call's first step: B half a step on, the current cleared.
+cudaError_t enqueue_start(pic_batch *b)
+{
+    k_b_yee_b<<<b->grid_stage, kBlock, 0, b->stream>>>(b->d_counts, b->d_runs, b->d_bm_cell,
+                                                       kYeeStart | kYeeZeroJ);
+    return cudaGetLastError();
+}
+
+// Launch sequence of one batch step on b->stream (also used while capturing); last: no step of
+// the same call follows.  Every grid is fixed by the capacities; the kernels read the table
+// lengths from d_counts.
+cudaError_t enqueue_step(pic_batch *b, bool last)
 {
     cudaStream_t st = b->stream;
     const Counts *cn = b->d_counts;
@@ -448,16 +442,15 @@ cudaError_t enqueue_step(pic_batch *b)
         k_b_swap<<<b->grid_runs, 128, 0, st>>>(cn, b->d_runs, b->d_due, s);
         nl += 8;
     }
-    k_b_zero_j<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell);
-    ++nl;
     if (b->timing) cudaEventRecord(b->ev0, st);
     k_b_gpp<<<b->grid_gpp, 256, b->smem, st>>>(cn, b->d_runs, b->d_state, b->d_items, b->d_counter);
     if (b->timing) cudaEventRecord(b->ev1, st);
     ++nl;
-    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, kYeeStart);
     k_b_yee_e<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell);
-    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(cn, b->d_runs, b->d_bm_cell, kYeeFinish | kYeeShadow);
-    nl += 3;
+    k_b_yee_b<<<b->grid_stage, kBlock, 0, st>>>(
+        cn, b->d_runs, b->d_bm_cell,
+        kYeeFinish | kYeeShadow | (last ? 0 : kYeeStart | kYeeZeroJ));
+    nl += 2;
     b->launches = nl;
     return cudaGetLastError();
 }
@@ -550,7 +543,7 @@ int pic_batch_create(pic_ctx *const *runs, int n, pic_batch **out)
     b->base = nullptr;
     b->bytes = 0;
     b->owns = false;
-    b->have_graph = false;
+    b->have_graph[0] = b->have_graph[1] = false;
     b->timing = false;
     b->steps_since_sync = 0;
     b->launches = 0;
@@ -690,28 +683,40 @@ int pic_batch_set_runs(pic_batch *b, pic_ctx *const *runs, int n)
     return upload(b, runs, n, t);
 }
 
+// The graph of a step, captured on first use (null: the capture failed).
+static cudaGraphExec_t step_graph(pic_batch *b, bool last)
+{
+    const int k = last ? 1 : 0;
+    if (!b->have_graph[k]) {
+        cudaGraph_t g;
+        if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        const cudaError_t e = enqueue_step(b, last);
+        if (cudaStreamEndCapture(b->stream, &g) != cudaSuccess || e != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        const cudaError_t ie = cudaGraphInstantiate(&b->exec[k], g, 0);
+        cudaGraphDestroy(g);
+        if (ie != cudaSuccess) return nullptr;
+        b->have_graph[k] = true;
+    }
+    return b->exec[k];
+}
+
 int pic_batch_step(pic_batch *b, int nsteps)
 {
     if (!b || nsteps < 0) return PIC_EINVAL;
     if (!b->base) return PIC_ESTATE;
-    if (!b->have_graph) {
-        cudaGraph_t g;
-        if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            cudaGetLastError();
-            return PIC_ECUDA;
-        }
-        const cudaError_t e = enqueue_step(b);
-        if (cudaStreamEndCapture(b->stream, &g) != cudaSuccess || e != cudaSuccess) {
-            cudaGetLastError();
-            return PIC_ECUDA;
-        }
-        const cudaError_t ie = cudaGraphInstantiate(&b->exec, g, 0);
-        cudaGraphDestroy(g);
-        if (ie != cudaSuccess) return PIC_ECUDA;
-        b->have_graph = true;
-    }
+    if (nsteps == 0) return PIC_OK;
+    cudaGraphExec_t mid = nullptr;
+    const cudaGraphExec_t last = step_graph(b, true);
+    if (!last || (nsteps > 1 && !(mid = step_graph(b, false)))) return PIC_ECUDA;
+    if (enqueue_start(b) != cudaSuccess) return PIC_ECUDA;
     for (int i = 0; i < nsteps; ++i)
-        if (cudaGraphLaunch(b->exec, b->stream) != cudaSuccess) return PIC_ECUDA;
+        if (cudaGraphLaunch(i + 1 < nsteps ? mid : last, b->stream) != cudaSuccess) return PIC_ECUDA;
     b->steps_since_sync += nsteps;
     return PIC_OK;
 }
@@ -723,7 +728,8 @@ int pic_batch_time_gpp(pic_batch *b, double *ms)
     if (!b || !ms) return PIC_EINVAL;
     if (!b->base) return PIC_ESTATE;
     b->timing = true;
-    const cudaError_t e = enqueue_step(b);
+    cudaError_t e = enqueue_start(b);
+    if (e == cudaSuccess) e = enqueue_step(b, true);
     b->timing = false;
     if (e != cudaSuccess) return PIC_ECUDA;
     b->steps_since_sync += 1;
@@ -765,7 +771,8 @@ void pic_batch_destroy(pic_batch *b)
         cudaEventDestroy(b->ev0);
         cudaEventDestroy(b->ev1);
     }
-    if (b->have_graph) cudaGraphExecDestroy(b->exec);
+    for (int k = 0; k < 2; ++k)
+        if (b->have_graph[k]) cudaGraphExecDestroy(b->exec[k]);
     if (b->owns && b->base) cudaFree(b->base);
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
