@@ -52,12 +52,11 @@ WORKLOAD = "pair_2048x1024_l3_WT_g50_uth0.01_ppc64_cdt0.25"
 # (fields read, current written), for the kernel-only view reported beside the roofline.
 BYTES = {"fp64": (80.0, 240.0), "fp32": (48.0, 310.0)}
 KERNEL_GRID_BYTES = {"fp64": 72.0, "fp32": 48.0}
-WEIGHT_CACHE_BYTES_FP64_L3 = 128.0
 SCHEDULERS_PER_SM = 4
 # The particle kernel's sources: the counts of profiles/counts.txt (from one ncu capture) are
 # used only while these files hash to the digest recorded with them.
 KERNEL_SOURCES = ("pic_common.cuh", "pic_gpp.cuh", "pic_gpp_kernels.cuh", "pic_gpp_f32.cu",
-                  "pic_gpp_f64.cu")
+                  "pic_gpp_f64.cu", "pic_gpp_fx.cuh", "pic_fixed.cuh")
 
 
 def _rank_env():
@@ -790,29 +789,16 @@ def main():
         fp64_peak = pic.pic_probe_fma_peak(0)
     except Exception:
         pass
-    hbm_view = {"achieved_gbs": alg_bytes / gpp_avg_s / 1e9,
-                "frac_of_measured_hbm": alg_bytes / gpp_avg_s / 1e9 / peaks["hbm_gbs"],
-                "weight_cache_bytes_per_particle": WEIGHT_CACHE_BYTES_FP64_L3,
-                "traffic_over_algorithmic": (traffic64 / alg_bytes) if traffic64 else None,
-                "note": "the DRAM traffic includes the read and write of the cached B-spline "
-                        "weights (128 B per particle-step), bytes spent to save FP64 "
-                        "instructions in a form bound by its FP64 pipe"}
-    flops = c64.get("fp64_flops_per_particle")
-    if flops and fp64_peak:
-        ach = res["n"] * flops / gpp_avg_s / 1e12
-        roofline = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s",
-                    "frac": ach / fp64_peak, "traffic": traffic64,
-                    "peak_source": "measured FP64 FMA rate (pic_probe_fma_peak, all SMs)",
-                    "flops_per_particle": flops,
-                    "fp64_instr_frac": (res["n"] * c64.get("fp64_instr_per_particle", 0.0) / gpp_avg_s)
-                                       / (fp64_peak * 1e12 / 2.0),
-                    "hbm_view": hbm_view}
-    else:
-        ach = alg_bytes / gpp_avg_s / 1e9
-        roofline = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                    "frac": ach / peaks["hbm_gbs"], "traffic": traffic64,
-                    "peak_source": "%s hbm_gbs" % peak_kind,
-                    "note": "no FP64 instruction count recorded for these kernel sources"}
+    ach = alg_bytes / gpp_avg_s / 1e9
+    roofline = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": ach / peaks["hbm_gbs"], "traffic": traffic64,
+                "peak_source": "%s hbm_gbs" % peak_kind,
+                "note": "bound on chip: the weights, gather and current products run on the "
+                        "integer units in 62-bit fixed point, the push on the FP64 pipe"}
+    instr = c64.get("fp64_pipe_instr_per_particle")
+    if instr and fp64_peak:  # the FP64 pipe completes peak / 2 instructions per second
+        roofline["fp64_pipe_frac"] = res["n"] * instr / gpp_avg_s / (fp64_peak * 1e12 / 2.0)
+        roofline["warp_instr_per_particle"] = c64.get("warp_instr_per_particle")
     roofline["kernel"] = "k_gpp2d<3,4> (double): fused gather+push+move+deposit"
     roofline["kernel_ms"] = gpp_avg_s * 1e3
     roofline["algorithmic_bytes"] = alg_bytes
