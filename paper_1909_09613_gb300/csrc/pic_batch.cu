@@ -37,6 +37,7 @@ int ctx_prepare_batch(pic_ctx *c);
 int ctx_sort_interval(const pic_ctx *c);
 int ctx_age(const pic_ctx *c);
 cudaStream_t ctx_stream(const pic_ctx *c);
+int32_t *ctx_err_word(const pic_ctx *c);
 bool ctx_bound(const pic_ctx *c);
 }  // namespace pic
 
@@ -471,12 +472,17 @@ int write_back(pic_batch *b, int32_t *err_out)
             return PIC_ECUDA;
         for (int r = 0; r < b->n; ++r)
             ctx_after_batch(b->ctx[r], rds[r], sts[r].age, b->steps_since_sync);
+        // the runs' error words: all copies, then one wait
+        std::vector<int32_t> words(b->n);
         for (int r = 0; r < b->n; ++r) {
-            int32_t e = 0;
-            if (cudaMemcpy(&e, rds[r].err, sizeof(e), cudaMemcpyDeviceToHost) != cudaSuccess)
+            int32_t *at = ctx_err_word(b->ctx[r]) ? ctx_err_word(b->ctx[r]) : &words[r];
+            if (cudaMemcpyAsync(at, rds[r].err, sizeof(*at), cudaMemcpyDeviceToHost, b->stream)
+                != cudaSuccess)
                 return PIC_ECUDA;
-            err |= e;
         }
+        if (cudaStreamSynchronize(b->stream) != cudaSuccess) return PIC_ECUDA;
+        for (int r = 0; r < b->n; ++r)
+            err |= ctx_err_word(b->ctx[r]) ? *ctx_err_word(b->ctx[r]) : words[r];
     }
     b->steps_since_sync = 0;
     if (err_out) *err_out = err;
