@@ -7,7 +7,7 @@ namespace pic {
 namespace {
 
 template <int L, int KT, bool DET>
-__global__ void __launch_bounds__(256, 2) k_gpp2d(const __grid_constant__ RunDev rd)
+__global__ void __launch_bounds__(32 * fx_warps(L), 2) k_gpp2d(const __grid_constant__ RunDev rd)
 {
     extern __shared__ __align__(16) char smem[];
     tile_fx<L, KT, DET>(rd, smem, blockIdx.x);
@@ -20,7 +20,7 @@ cudaError_t go(const RunDev &rd, cudaStream_t st)
     auto k = rd.det ? k_gpp2d<L, KT, true> : k_gpp2d<L, KT, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3((unsigned)rd.ntiles, tile_parts(rd)), 256, smem, st>>>(rd);
+    k<<<dim3((unsigned)rd.ntiles, tile_parts(rd)), 32 * fx_warps(L), smem, st>>>(rd);
     return cudaGetLastError();
 }
 

@@ -25,6 +25,11 @@ struct StageFx {
     int *emax;  // exponent field of the largest magnitude, per component (E1..E3, B1..B3)
 };
 
+// Warps of a block, two blocks per SM.  Quartic splines spill at the 128 registers of 16 warps per
+// SM as they do at the 96 of 20, and the extra warps hide more of the wait (255x130 at 16 per cell
+// 338 -> 316 us); cubic ones do not spill and lose (134M particles 40.7 -> 42.5 ms).
+__host__ __device__ constexpr int fx_warps(int l) { return l == 4 ? 10 : 8; }
+
 constexpr int kFxHead = 2 * sizeof(TTable) + 32;  // tables and exponents
 
 __host__ __device__ inline size_t stage_fx_bytes(int64_t nodes)
@@ -54,6 +59,7 @@ __device__ __forceinline__ uint2 field_limbs(double f, int emax)
 // Stage the fields of the tile at (x0, y0): the largest exponent of every component over the
 // staged region first, then the fields in its units (the second read comes from L1 or L2).
 // One warp per row.
+template <int W>
 __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0, int y0)
 {
     const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -62,7 +68,7 @@ __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0
     if (threadIdx.x < 6) st.emax[threadIdx.x] = 0;
     __syncthreads();
     int em[6] = {0, 0, 0, 0, 0, 0};
-    for (int ry = warp; ry < RY; ry += kTileWarps) {
+    for (int ry = warp; ry < RY; ry += W) {
         const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
         for (int rx = lane; rx < RX; rx += 32) {
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
@@ -79,7 +85,7 @@ __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < 6; ++c) em[c] = st.emax[c];
-    for (int ry = warp; ry < RY; ry += kTileWarps) {
+    for (int ry = warp; ry < RY; ry += W) {
         const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
         for (int rx = lane; rx < RX; rx += 32) {
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
@@ -397,10 +403,11 @@ __device__ __forceinline__ void particle_fx(const Hot2D &h, const HotSp<double> 
 template <int L, int KT, bool DET>
 __device__ void tile_fx(const RunDev &rd, char *smem, int64_t tile)
 {
+    constexpr int W = fx_warps(L);
     const StageFx st = stage_fx_carve(smem, (int)rd.reg_nodes);
     const int tx = (int)(tile % rd.ntile[0]), ty = (int)(tile / rd.ntile[0]);
     const int x0 = tx * rd.tile[0], y0 = ty * rd.tile[1];
-    stage_fx_load(rd, st, x0, y0);
+    stage_fx_load<W>(rd, st, x0, y0);
     const Hot2D h = make_hot2d(rd);
     __syncthreads();
     for (int s = 0; s < rd.nsp; ++s) {
@@ -411,7 +418,7 @@ __device__ void tile_fx(const RunDev &rd, char *smem, int64_t tile)
         // warp-uniform trip count: a warp's lanes take 32 consecutive particles.  The species
         // start at different warps, so that a part of few particles does not queue its species
         // one behind the other on the first warps.
-        const int w = ((threadIdx.x >> 5) + s * (kTileWarps / 2)) % kTileWarps;
+        const int w = ((threadIdx.x >> 5) + s * (W / 2)) % W;
         for (int64_t q = a + 32 * w; q < b; q += blockDim.x) {
             const int64_t p = q + (threadIdx.x & 31);
             if (p + blockDim.x < b) prefetch_particle<double>(hs, p + blockDim.x);
