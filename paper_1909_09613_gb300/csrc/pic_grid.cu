@@ -633,7 +633,13 @@ static cudaError_t launch_rho(const RunDev &rd, double *rho, cudaStream_t st)
     if (n == 0) return cudaSuccess;
     int sh = 0;
     while (!rd.slot_major && sh < 5 && (rd.ncell << (sh + 1)) <= n) ++sh;
-    const RhoWin win = rho_window(rd);
+    RhoWin win = rho_window(rd);
+    // zeroing and adding the window costs as much as what it saves below about eight
+    // contributions per node (FP64 96x40x36 quadratic, 4 of a species per cell: 4.8 per node, pic_diag
+    // 263 us without a window, 298 with; FP32 256x64x64 alike: 10.4 per node, 1120 and 1057)
+    double sums = (double)n / rd.ntiles;
+    for (int a = 0; a < rd.dim; ++a) sums *= rd.l + 1;
+    if (sums < 8.0 * win.nodes) win.nodes = 0;
     // parts of a tile: enough blocks for a grid of few tiles, each of a thousand particles or more
     const int64_t want = (2048 + rd.ntiles - 1) / rd.ntiles, most = n / rd.ntiles / 1024;
     const int64_t parts = want < most ? want : most;
