@@ -849,7 +849,7 @@ int pic_step(pic_ctx *c, int nsteps)
     if (rd.det) set_det_scale(c);
     // B half a step ahead, B at integer time kept for the gather, the current cleared
     if (nsteps > 0) {
-        if (launch_yee_b(rd, true, false, c->stream) != cudaSuccess) return PIC_ECUDA;
+        if (launch_yee_start(rd, c->stream) != cudaSuccess) return PIC_ECUDA;
         c->kernel_launches += 1;
     }
     for (int it = 0; it < nsteps; ++it) {
@@ -878,9 +878,8 @@ int pic_step(pic_ctx *c, int nsteps)
             if (launch_j32_finish(rd, c->stream) != cudaSuccess) return PIC_ECUDA;
             c->kernel_launches += 1;
         }
-        if (launch_yee_e(rd, shadow, c->stream) != cudaSuccess) return PIC_ECUDA;
-        if (launch_yee_b(rd, false, it + 1 == nsteps, c->stream) != cudaSuccess) return PIC_ECUDA;
-        c->kernel_launches += 3;
+        if (launch_yee_step(rd, shadow, it + 1 == nsteps, c->stream) != cudaSuccess) return PIC_ECUDA;
+        c->kernel_launches += 1 + yee_step_launches(rd);
         c->age += 1;
         c->step += 1;
     }

@@ -75,8 +75,11 @@ cudaError_t launch_gpp3d(const RunDev &rd, int kt, cudaStream_t st);
 size_t gpp3d_smem_bytes(const RunDev &rd);
 
 // Yee and grid kernels
-cudaError_t launch_yee_b(const RunDev &rd, bool first, bool last, cudaStream_t st);
-cudaError_t launch_yee_e(const RunDev &rd, bool shadow, cudaStream_t st);
+// ahead of a call's first step: B half a step on, the current cleared
+cudaError_t launch_yee_start(const RunDev &rd, cudaStream_t st);
+// after the particle pass: E, then B to integer time (last step of a call) or half a step past it
+cudaError_t launch_yee_step(const RunDev &rd, bool shadow, bool last, cudaStream_t st);
+int yee_step_launches(const RunDev &rd);
 cudaError_t launch_shadow(const RunDev &rd, cudaStream_t st);
 
 // particle packing (load / read back)
