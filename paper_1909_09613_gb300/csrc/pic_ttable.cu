@@ -134,8 +134,11 @@ static ld breakpoint(int scheme, ld dtt)
 // The fixed-point form of a table (the FP64 form of a run) from its Taylor coefficients.
 static void fix_table(int l, ld R, ld phib, const ld (*c)[PIC_TK_MAX][5], TTable *t)
 {
-    t->fx.rfrac = (uint64_t)std::ldexp(R - t->Rint, 64);
-    t->fx.phib = (uint64_t)std::ldexp(phib, 64);
+    // Rint is the floor of R as a double, which rounds up to the next integer where R lies less than
+    // half an ulp below it: the fraction is then negative, down to -2^-52, and counts as zero
+    const ld frac = R - t->Rint;
+    t->fx.rfrac = frac > 0 ? (uint64_t)std::ldexp(frac, 64) : 0;
+    t->fx.phib = (uint64_t)std::ldexp(phib, 64);  // breakpoint() gives 0 or a value inside (0, 1)
     for (int p = 0; p < 2; ++p) {
         const ld h = p ? 1 - phib : (phib > 0 ? phib : 1);
         // 2^shift <= 1 / h < 2^(shift + 1)
