@@ -190,10 +190,15 @@ __device__ __forceinline__ void particle3_fx(const RunDev &rd, const SpeciesDev 
     }
     if (!act) return;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)  // a non-finite velocity is reported as such, at the first node
-        if ((__double2hiint(dl[a]) & 0x7ff00000) == 0x7ff00000)
+    for (int a = 0; a < 3; ++a) {
+        // a non-finite velocity is reported as such, at the first node (a deterministic run's
+        // current holds integers: in the error word)
+        if ((__double2hiint(dl[a]) & 0x7ff00000) != 0x7ff00000) continue;
+        if (DET) set_err(rd.err, 2);
+        else
             atomicAdd(rd.F[6 + a] + (wrap_near(g0[2], rd.n[2]) * rd.n[1] + wrap_near(g0[1], rd.n[1])) * rd.n[0]
                           + wrap_near(g0[0], rd.n[0]), dl[a]);
+    }
     deposit3_fx<L, DET>(rd, sp, g0, S, up, mv);
 
     // ---- store ----

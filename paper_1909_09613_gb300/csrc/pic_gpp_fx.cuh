@@ -382,8 +382,10 @@ __device__ __forceinline__ void particle_fx(const Hot2D &h, const HotSp<double> 
     double kz = hs.kz * u[2] * ig;
     const int gx0 = x0 - h.pre0 + sx + Sx.wb, gy0 = y0 - h.pre1 + sy + Sy.wb;
     if (act && (__double2hiint(kz) & 0x7ff00000) == 0x7ff00000) {
-        // a non-finite velocity: its current is reported as such, at the first node
-        atomicAdd(h.J2 + (int64_t)wrap_near(gy0, h.n1) * h.n0 + wrap_near(gx0, h.n0), kz);
+        // a non-finite velocity: its current is reported as such, at the first node; a deterministic
+        // run's current holds integers and reports it in the error word
+        if (DET) set_err(h.err, 2);
+        else atomicAdd(h.J2 + (int64_t)wrap_near(gy0, h.n1) * h.n0 + wrap_near(gx0, h.n0), kz);
         kz = 0.0;
     }
     // a drift along x1 rarely moves the y window: skip its empty last row warp-uniformly
