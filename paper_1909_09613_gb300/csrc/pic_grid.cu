@@ -31,17 +31,20 @@ __global__ void __launch_bounds__(kBlock) k_yee_e(const __grid_constant__ RunDev
 // Both updates of a step of a small grid in one launch: one cluster of kYeeCtas blocks takes E, then
 // (cluster barrier: B reads E of the neighbouring cells, other blocks' among them) B.  Two launches
 // of a few blocks are 5 us each, nearly all of it launch and first loads (50 steps of 64x32 cells:
-// 1960 -> 1843 us in the FP64 form, 1747 -> 1695 in the FP32 form).
+// 1960 -> 1843 us in the FP64 form, 1747 -> 1695 in the FP32 form).  Up to one cell per thread: a
+// second one waits for the FP64 pipes of the eight SMs while two launches have more of them (50
+// steps, two launches -> cluster, us: 2,048 cells Yee 2018 -> 1970, M4 2328 -> 2185, 3D M4 6442 ->
+// 6290; 3,072 cells Yee 2328 -> 2384, M4 2635 -> 2810; 4,096 cells M4 2668 -> 2854, 3D 6485 -> 6879).
 constexpr int kYeeCtas = 8;
-constexpr int64_t kYeeOneCells = 4096;  // above, the FP64 pipes of eight SMs take as long
+constexpr int64_t kYeeOneCells = kYeeCtas * kBlock;
 
 __global__ void __cluster_dims__(kYeeCtas, 1, 1) __launch_bounds__(kBlock)
 k_yee_eb(const __grid_constant__ RunDev rd, double h, int shadow, int flags)
 {
-    const int first = blockIdx.x * kBlock + threadIdx.x;
-    for (int64_t c = first; c < rd.ncell; c += kYeeCtas * kBlock) yee_e_cell(rd, c, shadow);
+    const int c = blockIdx.x * kBlock + threadIdx.x;
+    if (c < rd.ncell) yee_e_cell(rd, c, shadow);
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-    for (int64_t c = first; c < rd.ncell; c += kYeeCtas * kBlock) yee_b_cell(rd, c, h, flags);
+    if (c < rd.ncell) yee_b_cell(rd, c, h, flags);
 }
 
 __global__ void __launch_bounds__(kBlock) k_shadow(const __grid_constant__ RunDev rd)
