@@ -140,9 +140,11 @@ __device__ __forceinline__ Stage2D<R> stage2d_carve(char *smem, int64_t nodes,
 // remainders per node, which paced the small runs: 64x32 cells 23.4 -> 17.8 us per
 // pass, 250x126 44.7 -> 42.7, the batch of 48 uneven runs 2.60 -> 2.51 ms).
 template <typename R>
-__device__ void stage2d_load(const RunDev &rd, const Stage2D<R> &st, int x0, int y0)
+__device__ void stage2d_load(const RunDev &rd, const Stage2D<R> &st, int x0, int y0, int tiles)
 {
     const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < (tiles - 1) * 3 * RX * RY / 2; i += blockDim.x)
+        ((float2 *)st.rec)[i] = make_float2(0.0f, 0.0f);
     if (st.tt != rd.tt)
         for (int i = threadIdx.x; i < (int)(2 * sizeof(TTable) / sizeof(int)); i += blockDim.x)
             ((int *)st.tt)[i] = ((const int *)rd.tt)[i];
@@ -171,26 +173,61 @@ __device__ void stage2d_load(const RunDev &rd, const Stage2D<R> &st, int x0, int
     }
 }
 
-// Add the current tile to the global FP64 current.  One warp per row, as stage2d_load.
+// Current tiles of a CTA.  A deterministic run sums integers, exact in any order: one tile for all
+// species.  Otherwise the species are added to each other in FP64 only (a neutral plasma's currents
+// cancel, and their sum in FP32 would be rounded at the size of one species' current): in the
+// slot-major order, which writes no deposit records, every species has a tile of its own, the
+// further ones where the records would lie, if they fit; else one tile is flushed once per species.
+// (One FP32 tile and one flush for all species is faster by what the second flush takes, us per pass:
+// 64x32 quadratic at 2 of a species per cell 17.6 against 19.7 (24.2 with the tiles added in the SM);
+// 250x126 cubic at 4 52.6 against 56.2; 512x256 cubic at 16 283 against 294.)
+template <int L, bool DET>
+__device__ __forceinline__ int current_tiles(const RunDev &rd)
+{
+    const bool fit = (rd.nsp - 1) * 3 * rd.reg_nodes <= kTileWarps * (int64_t)dep_record_floats(L);
+    return !DET && rd.slot_major && fit ? rd.nsp : 1;
+}
+
+// Add the current tiles to the global FP64 current; clear: and zero them for another species.  One
+// warp per row, two neighbouring nodes per lane (rows hold an even number of nodes).
 template <typename R>
-__device__ void stage2d_flush(const RunDev &rd, const Stage2D<R> &st, int x0, int y0)
+__device__ void stage2d_flush(const RunDev &rd, const Stage2D<R> &st, int x0, int y0, int tiles,
+                              bool clear)
 {
     const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31;
+    const int nodes = RX * RY;
     for (int ry = threadIdx.x >> 5; ry < RY; ry += kTileWarps) {
         const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
-        for (int rx = lane; rx < RX; rx += 32) {
-            const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
+        for (int rx = 2 * lane; rx < RX; rx += 64) {
+            const int64_t g0 = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
+            const int64_t g1 = row + wrap_near(x0 - rd.pre[0] + rx + 1, rd.n[0]);
             const int n = ry * RX + rx;
-            if (st.q1) {  // deterministic run: integer sums, exact in any order
-                const unsigned long long a = st.q1[n], b = st.q2[n], c = st.q3[n];
-                if (a) atomicAdd((unsigned long long *)(rd.F[6] + g), a);
-                if (b) atomicAdd((unsigned long long *)(rd.F[7] + g), b);
-                if (c) atomicAdd((unsigned long long *)(rd.F[8] + g), c);
-            } else {
-                const R a = st.j1[n], b = st.j2[n], c = st.j3[n];
-                if (a != R(0)) atomicAdd(rd.F[6] + g, (double)a);
-                if (b != R(0)) atomicAdd(rd.F[7] + g, (double)b);
-                if (c != R(0)) atomicAdd(rd.F[8] + g, (double)c);
+            if (st.q1) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    unsigned long long *q = i == 0 ? st.q1 : (i == 1 ? st.q2 : st.q3);
+                    unsigned long long *J = (unsigned long long *)rd.F[6 + i];
+                    const unsigned long long a = q[n], b = q[n + 1];
+                    if (a) atomicAdd(J + g0, a);
+                    if (b) atomicAdd(J + g1, b);
+                }
+                continue;
+            }
+            float2 v[3] = {*(float2 *)(st.j1 + n), *(float2 *)(st.j2 + n), *(float2 *)(st.j3 + n)};
+            if (clear) {
+                const float2 z = make_float2(0.0f, 0.0f);
+                *(float2 *)(st.j1 + n) = *(float2 *)(st.j2 + n) = *(float2 *)(st.j3 + n) = z;
+            }
+            for (int k = 1;; ++k) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if (v[i].x != 0.0f) atomicAdd(rd.F[6 + i] + g0, (double)v[i].x);
+                    if (v[i].y != 0.0f) atomicAdd(rd.F[6 + i] + g1, (double)v[i].y);
+                }
+                if (k >= tiles) break;
+                const float *j = st.rec + (k - 1) * 3 * nodes + n;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) v[i] = *(const float2 *)(j + i * nodes);
             }
         }
     }
@@ -797,7 +834,9 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile, const TTable
     const int tx = (int)(tile % rd.ntile[0]);
     const int ty = (int)(tile / rd.ntile[0]);
     const int x0 = tx * rd.tile[0], y0 = ty * rd.tile[1];
-    stage2d_load<R>(rd, st, x0, y0);
+    const int tiles = current_tiles<L, DET>(rd);
+    const bool once = DET || tiles == rd.nsp;  // one flush, after the last species
+    stage2d_load<R>(rd, st, x0, y0, tiles);
     const Hot2D h = make_hot2d(rd);
     __syncthreads();
     for (int s = 0; s < rd.nsp; ++s) {
@@ -805,29 +844,42 @@ __device__ void tile_2d(const RunDev &rd, char *smem, int64_t tile, const TTable
         const HotSp<R> hs = make_hotsp<R>(sp);
         int64_t a = sp.tile_start[tile], b = sp.tile_start[tile + 1];
         split_range(split, a, b);
+        if (a >= b) continue;  // (the whole CTA)
+        Stage2D<R> own = st;
+        if (s > 0 && tiles > 1) {
+            own.j1 = st.rec + (s - 1) * 3 * (int)rd.reg_nodes;
+            own.j2 = own.j1 + (int)rd.reg_nodes;
+            own.j3 = own.j2 + (int)rd.reg_nodes;
+        }
         // every warp takes a contiguous chunk of the tile's particles of this species (for a
         // uniform plasma in the cell-major order, one row of cells), so that the warps' frames,
         // a row apart, rarely race for the same nodes of the tile: 5.53 -> 5.38 ms on the
         // 134M-particle FP32 step (slot-major runs, whose lanes deposit one by one, lose about
-        // 5%; a runtime choice between the two loops cost the dense kernel more).  The species
-        // of a part of few particles start at different warps, so as not to queue one behind the
-        // other on the first warps.
+        // 5%; a runtime choice between the two loops cost the dense kernel more).  With
+        // one flush, the species of a part of few particles start at different warps, so as not to
+        // queue one behind the other on the first warps.
         const int lane = threadIdx.x & 31;
         const int64_t groups = (b - a + 31) / 32;
-        const int w = ((threadIdx.x >> 5) + (groups < kTileWarps ? s * (kTileWarps / 2) : 0)) % kTileWarps;
+        const int w = ((threadIdx.x >> 5) + (once && groups < kTileWarps ? s * (kTileWarps / 2) : 0)) % kTileWarps;
         const int64_t gw = (groups + kTileWarps - 1) / kTileWarps;
         const int64_t ca = a + 32 * min(groups, (int64_t)w * gw);
         const int64_t cb = min(b, a + 32 * min(groups, (int64_t)(w + 1) * gw));
         for (int64_t q = ca; q < cb; q += 32) {  // warp-uniform trip count
             const int64_t p = q + lane;
             if (p + 32 < cb) prefetch_particle<R>(hs, p + 32);
-            particle_2d<L, KT, R, DET>(h, hs, st, p, p < cb, x0, y0);
+            particle_2d<L, KT, R, DET>(h, hs, own, p, p < cb, x0, y0);
+        }
+        if (!once) {
+            const bool more = s + 1 < rd.nsp;
+            __syncthreads();
+            stage2d_flush<R>(rd, st, x0, y0, 1, more);
+            if (more) __syncthreads();
         }
     }
-    // one flush for all species (one per species doubled the tile's FP64 atomics and held the
-    // warps at two more barriers)
-    __syncthreads();
-    stage2d_flush<R>(rd, st, x0, y0);
+    if (once) {
+        __syncthreads();
+        stage2d_flush<R>(rd, st, x0, y0, tiles, false);
+    }
 }
 
 }  // namespace pic
