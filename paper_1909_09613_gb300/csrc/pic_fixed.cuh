@@ -6,7 +6,8 @@
 // Everything between the particle's offset and its current is bounded -- offsets, weights and
 // their products lie in [0, 1], and a tile's fields lie below their largest magnitude -- so
 // 62-bit fixed point carries it with more bits than FP64's 53, at three such products per
-// multiplication.  The Boris push and the move, whose range is open, stay in FP64.
+// multiplication.  The Boris push and the move, whose range is open, stay in FP64, and so does the
+// gather of a tile whose fields differ by more than the fixed point resolves (stage_fx_load).
 //
 // U62: an unsigned value in units of 2^-62 (1 is 2^62), split for multiplication into limbs of
 // 31 bits, v = h 2^31 + l.  A product drops l l' (below one unit) and truncates the rest: it is
@@ -45,12 +46,13 @@ PIC_HD uint64_t mul62(const Limbs &a, const Limbs &b)
     return wide_mul(a.h, b.h) + ((wide_mul(a.h, b.l) + wide_mul(a.l, b.h)) >> 31);
 }
 
-// a s with a signed (|a| <= 2^62) and s a U62 below 1
+// a s with a signed (|a| <= 2^62) and s a U62 below 1; the constant makes up for the dropped l l' (on
+// average a quarter of a unit) and rounds, so that a chain of products has no one-signed error
 PIC_HD int64_t mul62s(int64_t a, const Limbs &s)
 {
     const int32_t ah = (int32_t)(a >> 31);
     const uint32_t al = (uint32_t)a & 0x7fffffffu;
-    const int64_t x = (int64_t)ah * (int32_t)s.l + (int64_t)wide_mul(al, s.h);
+    const int64_t x = (int64_t)ah * (int32_t)s.l + (int64_t)wide_mul(al, s.h) + 3 * (1 << 29);
     return (int64_t)ah * (int32_t)s.h + (x >> 31);
 }
 
@@ -216,17 +218,56 @@ __device__ __forceinline__ void red_fixed(double *p, uint64_t v, uint32_t top)
 }
 #endif
 
-// A field value as biased fixed point for a tile whose largest magnitude has the exponent field
-// emax: round(F 2^(59 - E)) + 2^59 with |F| < 2^E, E = emax - 1022.
-PIC_HD uint64_t field_fixed(uint64_t bits, int emax)
+// The FP64 value of a U62, rounded to nearest, by its bits.
+PIC_HD uint64_t weight_bits(uint64_t v) { return v ? to_fp64_bits(v, 1023u << 20) : 0; }
+
+// A signed value split for the gather's products, v = h 2^32 + l with |l| <= 2^31: the dropped l l'
+// have no sign of their own.
+struct Parts {
+    int32_t h, l;
+};
+
+PIC_HD Parts parts(int64_t v)
+{
+    Parts r;
+    r.l = (int32_t)(uint32_t)v;
+    r.h = (int32_t)((uint64_t)v >> 32) + (r.l < 0 ? 1 : 0);
+    return r;
+}
+
+// Sum of weight x field products, weights U62 (as Parts) that sum to 1 and fields of at most 2^60
+// units: the high products and the cross products apart, so that a term costs three multiply-adds.
+// Bounds for up to six terms: hi below 2^59, x below 2.5 2^61.  A field of zeros sums to zero exactly,
+// and the rounding of the others (about one unit) has no sign of its own.
+struct GatherSum {
+    int64_t hi, x;
+    PIC_HD void zero() { hi = 0; x = 1 << 29; }  // (half of what value() shifts out)
+    PIC_HD void add(const Parts &w, int32_t fh, int32_t fl)
+    {
+        hi += (int64_t)w.h * fh;
+        x += (int64_t)w.h * fl;
+        x += (int64_t)w.l * fh;
+    }
+    PIC_HD int64_t value() const { return 4 * hi + (x >> 30); }
+};
+
+// A field value in the fixed point of a tile whose largest magnitude has the exponent field emax:
+// round(F 2^(60 - E)) with |F| < 2^E, E = emax - 1022.  Only zero gives zero: a value below half a
+// unit gives one unit of its sign.
+PIC_HD int64_t field_fixed(uint64_t bits, int emax)
 {
     const int e = (int)(bits >> 52) & 0x7ff;
-    const uint64_t m = e == 0 ? 0 : ((bits & 0xfffffffffffffull) | ((uint64_t)1 << 52)) << 6;
+    const uint64_t f = bits & 0xfffffffffffffull;
+    const uint64_t m = e == 0 ? 0 : (f | ((uint64_t)1 << 52)) << 7;
     const int r = emax - e;
-    const uint64_t v = r > 60 ? 0 : (r > 0 ? ((m >> (r - 1)) + 1) >> 1 : m);
-    const uint64_t one = (uint64_t)1 << 59;
-    return (bits >> 63) ? one - v : one + v;
+    uint64_t v = r > 61 ? 0 : (r > 0 ? ((m >> (r - 1)) + 1) >> 1 : m);
+    if (v == 0 && (e | (f != 0)) != 0) v = 1;
+    return (bits >> 63) ? -(int64_t)v : (int64_t)v;
 }
+
+// One unit of the gather is at most one FP64 rounding of the largest field in a stencil that holds a
+// field of 2^53 units or more, one whose exponent field is less than kSmallField below emax.
+constexpr int kSmallField = 7;
 
 // Esirkepov window of one axis in U62: weights of the old (s0) and the new position (s1) on
 // l + 2 nodes starting at node wb relative to the old cell (AxisS in fixed point).

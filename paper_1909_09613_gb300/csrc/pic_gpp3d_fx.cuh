@@ -36,12 +36,6 @@ __device__ __forceinline__ double gather3_global(const double *f, int nx, int ny
     return acc;
 }
 
-// The FP64 value of a U62, rounded to nearest, by its bits.
-__device__ __forceinline__ double weight_value(uint64_t v)
-{
-    return v ? __longlong_as_double((int64_t)to_fp64_bits(v, 1023u << 20)) : 0.0;
-}
-
 // The Esirkepov window of one particle added to the global FP64 current (reductions performed by
 // L2).  With S0, S1 the old and new weights of an axis, P the prefix sums of S1 - S0 and (a, b, c)
 // the axes in cyclic order,

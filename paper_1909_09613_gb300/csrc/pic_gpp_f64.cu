@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(32 * fx_warps(L), 2) k_gpp2d(const __grid_cons
 template <int L, int KT>
 cudaError_t go(const RunDev &rd, cudaStream_t st)
 {
-    const size_t smem = stage_fx_bytes(rd.reg_nodes);
+    const size_t smem = stage_fx_launch_bytes(rd);
     auto k = rd.det ? k_gpp2d<L, KT, true> : k_gpp2d<L, KT, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

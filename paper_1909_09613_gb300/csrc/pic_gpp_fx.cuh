@@ -9,20 +9,30 @@
 // 2.70 ms per pass over 8.4 M particles; 255x130, quartic, 16 per cell: 0.72 -> 0.34 ms.  Three
 // CTAs per SM at 80 registers spill (2.90 ms).  The old-position weights, which the FP64
 // evaluation read from a per-particle cache (128 B per particle and step), are evaluated.
+//
+// The gather's signed, rounded sums and the search for tiles whose fields one scale does not resolve
+// cost 6% of it (512x256, cubic, 32 of a species per cell, 8.4 M particles: 3.11 -> 3.32 ms; 64x32 at
+// 8: 37.6 -> 41.3 us, most of it the search) against biased sums of truncated products, which gave a
+// particle a one-signed field of 2^-54 of the tile's largest where its own was zero, and a node below
+// 2^-6 of the largest fewer bits than FP64.
 #pragma once
 #include "pic_fixed.cuh"
 #include "pic_gpp_kernels.cuh"
 
 namespace pic {
 
-// Shared-memory layout of a staged tile: biased fixed-point fields (field_fixed, units of
-// 2^(E - 59) with 2^E above the component's largest magnitude in the tile) split into limbs.
-//   pa = (E1, B2), pb = (E2, B1) as limb pairs (16 bytes), e3, b3 (8 bytes)
+// Shared-memory layout of a staged tile: the fields in fixed point (field_fixed, units of 2^(E - 60)
+// with 2^E above the component's largest magnitude in the tile) as Parts, or, in an exact tile, in
+// FP64.
+//   pa = (E1, B2), pb = (E2, B1) (16 bytes a node), e3, b3 (8 bytes), then the masks of small
+//   fields (mask_words)
 struct StageFx {
     uint4 *pa, *pb;
     uint2 *e3, *b3;
     TTable *tt;
-    int *emax;  // exponent field of the largest magnitude, per component (E1..E3, B1..B3)
+    int *emax;   // high word of the largest magnitude, per component (E1..E3, B1..B3)
+    int *exact;  // the tile's fields are staged in FP64 and gathered in FP64
+    uint32_t *mask;
 };
 
 // Warps of a block, two blocks per SM.  Quartic splines spill at the 128 registers of 16 warps per
@@ -30,42 +40,113 @@ struct StageFx {
 // 338 -> 316 us); cubic ones do not spill and lose (134M particles 40.7 -> 42.5 ms).
 __host__ __device__ constexpr int fx_warps(int l) { return l == 4 ? 10 : 8; }
 
-constexpr int kFxHead = 2 * sizeof(TTable) + 32;  // tables and exponents
+constexpr int kFxHead = 2 * sizeof(TTable) + 32;  // tables, exponents and the exact flag
 
 __host__ __device__ inline size_t stage_fx_bytes(int64_t nodes)
 {
     return (kFxHead + 15) / 16 * 16 + (size_t)nodes * 48;
 }
 
-__device__ __forceinline__ StageFx stage_fx_carve(char *smem, int nodes)
+// Words of the masks of small fields: per component and row one bit a node, set where it is small or
+// zero.
+__host__ __device__ inline int64_t mask_words(const RunDev &rd)
 {
+    return 6 * (int64_t)rd.reg[1] * ((rd.reg[0] + 31) / 32);
+}
+
+// Shared memory of a launch: with the masks where the device has room for them (without them every
+// tile is exact).
+__host__ __device__ inline size_t stage_fx_launch_bytes(const RunDev &rd)
+{
+    const size_t b = stage_fx_bytes(rd.reg_nodes), m = b + 4 * mask_words(rd);
+    return m <= 227 * 1024 ? m : b;
+}
+
+__device__ __forceinline__ StageFx stage_fx_carve(char *smem, const RunDev &rd)
+{
+    const size_t nodes = rd.reg_nodes;
     StageFx s;
     s.tt = (TTable *)smem;
     s.emax = (int *)(smem + 2 * sizeof(TTable));
+    s.exact = s.emax + 6;
     char *p = smem + (kFxHead + 15) / 16 * 16;
-    s.pa = (uint4 *)p; p += (size_t)nodes * 16;
-    s.pb = (uint4 *)p; p += (size_t)nodes * 16;
-    s.e3 = (uint2 *)p; p += (size_t)nodes * 8;
-    s.b3 = (uint2 *)p;
+    s.pa = (uint4 *)p; p += nodes * 16;
+    s.pb = (uint4 *)p; p += nodes * 16;
+    s.e3 = (uint2 *)p; p += nodes * 8;
+    s.b3 = (uint2 *)p; p += nodes * 8;
+    s.mask = stage_fx_launch_bytes(rd) > stage_fx_bytes(nodes) ? (uint32_t *)p : nullptr;
     return s;
 }
 
-__device__ __forceinline__ uint2 field_limbs(double f, int emax)
+__device__ __forceinline__ double field_at(const RunDev &rd, int c, int64_t g)
 {
-    const Limbs v = limbs(field_fixed((uint64_t)__double_as_longlong(f), emax));
-    return make_uint2(v.h, v.l);
+    return __ldg((c < 3 ? rd.F[c] : rd.Bg[c - 3]) + g);
 }
 
-// Stage the fields of the tile at (x0, y0): the largest exponent of every component over the
-// staged region first, then the fields in its units (the second read comes from L1 or L2).
-// One warp per row.
-template <int W>
+// A node's six fields into the stage, v(c) the 8 bytes of component c.
+template <typename V>
+__device__ __forceinline__ void stage_node(const StageFx &st, int n, const V &v)
+{
+    const uint2 e1 = v(0), e2 = v(1), b1 = v(3), b2 = v(4);
+    st.pa[n] = make_uint4(e1.x, e1.y, b2.x, b2.y);
+    st.pb[n] = make_uint4(e2.x, e2.y, b1.x, b1.y);
+    st.e3[n] = v(2);
+    st.b3[n] = v(5);
+}
+
+// Whether a staged field (fixed point) is zero, which field_fixed makes of zero alone.
+__device__ __forceinline__ bool staged_zero(const StageFx &st, int c, int n)
+{
+    const uint4 v = c == 0 || c == 4 ? st.pa[n] : st.pb[n];
+    if (c == 2 || c == 5) {
+        const uint2 w = c == 2 ? st.e3[n] : st.b3[n];
+        return (w.x | w.y) == 0;
+    }
+    return c < 2 ? (v.x | v.y) == 0 : (v.z | v.w) == 0;
+}
+
+// Whether some stencil of the tile may hold fields that are all small and not all zero: an
+// (L + 1) x (L + 1) window (no stencil is smaller) of small nodes with one that is not zero.
+// Thread by thread over component, row and mask word; components of zeros alone are left out.
+template <int L>
+__device__ __forceinline__ bool small_window(const RunDev &rd, const StageFx &st)
+{
+    const int RX = rd.reg[0], RY = rd.reg[1], mw = (RX + 31) / 32, rows = RY - L;
+    for (int i = threadIdx.x; i < 6 * rows * mw; i += blockDim.x) {
+        const int w = i % mw, ry = i / mw % rows, c = i / mw / rows;
+        if (st.emax[c] == 0) continue;
+        uint64_t s = ~(uint64_t)0;
+#pragma unroll
+        for (int k = 0; k <= L; ++k) {
+            const uint32_t *m = st.mask + (c * RY + ry + k) * mw + w;
+            s &= m[0] | (w + 1 < mw ? (uint64_t)m[1] << 32 : 0);
+        }
+        uint64_t all = s;  // bit b: the window of columns b .. b + L is small
+#pragma unroll
+        for (int k = 1; k <= L; ++k) all &= s >> k;
+        for (uint32_t left = (uint32_t)all; left; left &= left - 1) {
+            const int rx = 32 * w + __ffs(left) - 1;
+            for (int k = 0; k < (L + 1) * (L + 1); ++k)
+                if (!staged_zero(st, c, (ry + k / (L + 1)) * RX + rx + k % (L + 1))) return true;
+        }
+    }
+    return false;
+}
+
+// Stage the fields of the tile at (x0, y0): the largest exponent of every component over the staged
+// region first, then the fields in its units (the second read comes from L1 or L2).  One warp per row.
+// A unit is 2^-60 of the scale, so a stencil whose fields all lie below 2^-7 of it would be summed
+// with less than FP64's relative precision, and a non-finite or very small largest field gives no
+// scale: such a tile is staged again in FP64 and gathered in FP64 (st.exact).  Smooth and noisy fields
+// alike hold no such stencil (a window of l + 1 nodes squared crosses a zero, but is not that flat);
+// the edges of pulses and of regions without fields do.
+template <int L, int W>
 __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0, int y0)
 {
     const int RX = rd.reg[0], RY = rd.reg[1], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < (int)(2 * sizeof(TTable) / sizeof(int)); i += blockDim.x)
         ((int *)st.tt)[i] = ((const int *)rd.tt)[i];
-    if (threadIdx.x < 6) st.emax[threadIdx.x] = 0;
+    if (threadIdx.x < 7) st.emax[threadIdx.x] = 0;  // (exact among them)
     __syncthreads();
     int em[6] = {0, 0, 0, 0, 0, 0};
     for (int ry = warp; ry < RY; ry += W) {
@@ -73,80 +154,104 @@ __device__ inline void stage_fx_load(const RunDev &rd, const StageFx &st, int x0
         for (int rx = lane; rx < RX; rx += 32) {
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
 #pragma unroll
-            for (int c = 0; c < 6; ++c)
-                em[c] = max(em[c], __double2hiint(__ldg((c < 3 ? rd.F[c] : rd.Bg[c - 3]) + g)) & 0x7ff00000);
+            for (int c = 0; c < 6; ++c) {
+                const double f = field_at(rd, c, g);
+                em[c] = max(em[c], (__double2hiint(f) & 0x7fffffff) | (__double2loint(f) != 0 ? 1 : 0));
+            }
         }
     }
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
         const int m = __reduce_max_sync(0xffffffffu, em[c]);
-        if (lane == 0 && m > 0) atomicMax(st.emax + c, m >> 20);
+        if (lane == 0 && m > 0) atomicMax(st.emax + c, m);
     }
     __syncthreads();
+    bool exact = st.mask == nullptr;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) em[c] = st.emax[c];
+    for (int c = 0; c < 6; ++c) {
+        em[c] = st.emax[c];
+        exact = exact || em[c] >= 0x7ff00000 || (em[c] > 0 && em[c] < 64 << 20);
+        em[c] &= 0x7ff00000;
+    }
+    if (!exact) {
+        const int mw = (RX + 31) / 32;
+        for (int ry = warp; ry < RY; ry += W) {
+            const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
+            for (int w = 0; w < mw; ++w) {
+                const int rx = 32 * w + lane;
+                const bool in = rx < RX;
+                const int64_t g = row + wrap_near(x0 - rd.pre[0] + (in ? rx : 0), rd.n[0]);
+                uint32_t small[6];
+                uint2 p[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    const double f = field_at(rd, c, g);
+                    small[c] = __ballot_sync(0xffffffffu, in && (__double2hiint(f) & 0x7fffffff)
+                                                                    < em[c] - ((kSmallField - 1) << 20));
+                    const Parts q = parts(field_fixed((uint64_t)__double_as_longlong(f), em[c] >> 20));
+                    p[c] = make_uint2((uint32_t)q.h, (uint32_t)q.l);
+                }
+                if (in) stage_node(st, ry * RX + rx, [&](int c) { return p[c]; });
+                if (lane == 0) {
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) st.mask[(c * RY + ry) * mw + w] = small[c];
+                }
+            }
+        }
+        __syncthreads();
+        exact = __syncthreads_or(small_window<L>(rd, st));
+    }
+    if (!exact) return;
+    if (threadIdx.x == 0) *st.exact = 1;
     for (int ry = warp; ry < RY; ry += W) {
         const int64_t row = (int64_t)wrap_near(y0 - rd.pre[1] + ry, rd.n[1]) * rd.n[0];
         for (int rx = lane; rx < RX; rx += 32) {
             const int64_t g = row + wrap_near(x0 - rd.pre[0] + rx, rd.n[0]);
-            const int n = ry * RX + rx;
-            const uint2 e1 = field_limbs(__ldg(rd.F[0] + g), em[0]);
-            const uint2 b2 = field_limbs(__ldg(rd.Bg[1] + g), em[4]);
-            const uint2 e2 = field_limbs(__ldg(rd.F[1] + g), em[1]);
-            const uint2 b1 = field_limbs(__ldg(rd.Bg[0] + g), em[3]);
-            st.pa[n] = make_uint4(e1.x, e1.y, b2.x, b2.y);
-            st.pb[n] = make_uint4(e2.x, e2.y, b1.x, b1.y);
-            st.e3[n] = field_limbs(__ldg(rd.F[2] + g), em[2]);
-            st.b3[n] = field_limbs(__ldg(rd.Bg[2] + g), em[5]);
+            stage_node(st, ry * RX + rx, [&](int c) {
+                const double f = field_at(rd, c, g);
+                return make_uint2((uint32_t)__double2loint(f), (uint32_t)__double2hiint(f));
+            });
         }
     }
 }
 
-// Sum of weight x field products: the high products and the cross products apart, so that a
-// term costs three multiply-adds.  Bounds: the weights sum to 1 (2^62) and a field is below
-// 2^60, so hi stays below 2^60 and x below 2^62 + 6 2^60.
-struct AccFx {
-    uint64_t hi, x;
-    __device__ __forceinline__ void zero() { hi = 0; x = 0; }
-    __device__ __forceinline__ void add(const Limbs &w, uint32_t fh, uint32_t fl)
-    {
-        hi += wide_mul(w.h, fh);
-        x += wide_mul(w.h, fl);
-        x += wide_mul(w.l, fh);
-    }
-    __device__ __forceinline__ uint64_t value() const { return hi + (x >> 31); }
-};
-
-// The FP64 value of an interpolated biased field; emax as staged.  A tile with a non-finite
-// field gives NaN, a tile whose fields all lie below 2^-960 gives 0.
-__device__ __forceinline__ double field_value(uint64_t v, int emax)
+// The FP64 value of a weight.
+__device__ __forceinline__ double weight_value(uint64_t v)
 {
-    const double d = (double)((int64_t)v - ((int64_t)1 << 59));
-    const int e = emax - 1022 - 59 + 1023;  // exponent field of the unit
-    if (emax == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
-    return e <= 0 ? 0.0 : d * __hiloint2double(e << 20, 0);
+    return __longlong_as_double((int64_t)weight_bits(v));
 }
 
-// A pair of fields (first: limbs x, y; second: z, w) with weights wx along x, wy along y.
-template <int NX, int NY>
-__device__ __forceinline__ void gather_pair_fx(const uint4 *f, int RX, const Limbs *wx,
-                                               const Limbs *wy, uint64_t &a, uint64_t &b)
+__device__ __forceinline__ double weight_value(const Parts &w)
 {
-    AccFx A, B;
+    return weight_value((uint64_t)((int64_t)w.h * ((int64_t)1 << 32) + w.l));
+}
+
+// The FP64 value of an interpolated field; emax as staged, at least 64 << 20 (or a field of zeros).
+__device__ __forceinline__ double field_value(int64_t v, int emax)
+{
+    return (double)v * __hiloint2double((emax & 0x7ff00000) - ((60 - 1) << 20), 0);
+}
+
+// A pair of fields (first: parts x, y; second: z, w) with weights wx along x, wy along y.
+template <int NX, int NY>
+__device__ __forceinline__ void gather_pair_fx(const uint4 *f, int RX, const Parts *wx,
+                                               const Parts *wy, int64_t &a, int64_t &b)
+{
+    GatherSum A, B;
     A.zero();
     B.zero();
 #pragma unroll 1
     for (int j = 0; j < NY; ++j) {
-        AccFx ra, rb;
+        GatherSum ra, rb;
         ra.zero();
         rb.zero();
 #pragma unroll
         for (int i = 0; i < NX; ++i) {
             const uint4 v = f[j * RX + i];
-            ra.add(wx[i], v.x, v.y);
-            rb.add(wx[i], v.z, v.w);
+            ra.add(wx[i], (int)v.x, (int)v.y);
+            rb.add(wx[i], (int)v.z, (int)v.w);
         }
-        const Limbs la = limbs(ra.value()), lb = limbs(rb.value());
+        const Parts la = parts(ra.value()), lb = parts(rb.value());
         A.add(wy[j], la.h, la.l);
         B.add(wy[j], lb.h, lb.l);
     }
@@ -155,24 +260,43 @@ __device__ __forceinline__ void gather_pair_fx(const uint4 *f, int RX, const Lim
 }
 
 template <int NX, int NY>
-__device__ __forceinline__ uint64_t gather_one_fx(const uint2 *f, int RX, const Limbs *wx,
-                                                  const Limbs *wy)
+__device__ __forceinline__ int64_t gather_one_fx(const uint2 *f, int RX, const Parts *wx,
+                                                 const Parts *wy)
 {
-    AccFx A;
+    GatherSum A;
     A.zero();
 #pragma unroll 1
     for (int j = 0; j < NY; ++j) {
-        AccFx r;
+        GatherSum r;
         r.zero();
 #pragma unroll
         for (int i = 0; i < NX; ++i) {
             const uint2 v = f[j * RX + i];
-            r.add(wx[i], v.x, v.y);
+            r.add(wx[i], (int)v.x, (int)v.y);
         }
-        const Limbs l = limbs(r.value());
+        const Parts l = parts(r.value());
         A.add(wy[j], l.h, l.l);
     }
     return A.value();
+}
+
+// One field of an exact tile, in FP64: p its 8 bytes at the stencil's first node, stride those of a
+// node.
+template <int NX, int NY>
+__device__ __forceinline__ double gather_exact(const char *p, int stride, int RX, const Parts *wx,
+                                               const Parts *wy)
+{
+    double dx[NX], acc = 0.0;
+#pragma unroll
+    for (int i = 0; i < NX; ++i) dx[i] = weight_value(wx[i]);
+#pragma unroll 1
+    for (int j = 0; j < NY; ++j) {
+        double r = 0.0;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) r += dx[i] * *(const double *)(p + (size_t)(j * RX + i) * stride);
+        acc += weight_value(wy[j]) * r;
+    }
+    return acc;
 }
 
 // One contribution (v in U62, its scale's sign and exponent in top) added to a node of the
@@ -339,7 +463,7 @@ __device__ __forceinline__ void particle_fx(const Hot2D &h, const HotSp<double> 
     // ---- gather (Eq. interpolation-EB-real-mod; MC when the tables hold W_l) ----
     double E[3], B[3];
     {
-        Limbs wh[2][L + 1], wt[2][KT];
+        Parts wh[2][L + 1], wt[2][KT];
         int bh[2], bt[2];
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
@@ -348,21 +472,32 @@ __device__ __forceinline__ void particle_fx(const Hot2D &h, const HotSp<double> 
             bspline62<L>(psi, w);
             bt[a] = ttable_weights62<L, KT>(st.tt[a], f[a], t);
 #pragma unroll
-            for (int k = 0; k <= L; ++k) wh[a][k] = limbs(w[k]);
+            for (int k = 0; k <= L; ++k) wh[a][k] = parts((int64_t)w[k]);
 #pragma unroll
-            for (int k = 0; k < KT; ++k) wt[a][k] = limbs(t[k]);
+            for (int k = 0; k < KT; ++k) wt[a][k] = parts((int64_t)t[k]);
         }
         const int xh = sx + bh[0], xt = sx + bt[0];
         const int yh = (sy + bh[1]) * RX, yt = (sy + bt[1]) * RX;
-        uint64_t v[6];
-        gather_pair_fx<L + 1, KT>(st.pa + yt + xh, RX, wh[0], wt[1], v[0], v[4]);  // E1, B2
-        gather_pair_fx<KT, L + 1>(st.pb + yh + xt, RX, wt[0], wh[1], v[1], v[3]);  // E2, B1
-        v[2] = gather_one_fx<KT, KT>(st.e3 + yt + xt, RX, wt[0], wt[1]);
-        v[5] = gather_one_fx<L + 1, L + 1>(st.b3 + yh + xh, RX, wh[0], wh[1]);
+        const uint4 *pa = st.pa + yt + xh, *pb = st.pb + yh + xt;
+        const uint2 *p3 = st.e3 + yt + xt, *q3 = st.b3 + yh + xh;
+        if (*st.exact) {  // the whole CTA
+            E[0] = gather_exact<L + 1, KT>((const char *)pa, 16, RX, wh[0], wt[1]);
+            B[1] = gather_exact<L + 1, KT>((const char *)pa + 8, 16, RX, wh[0], wt[1]);
+            E[1] = gather_exact<KT, L + 1>((const char *)pb, 16, RX, wt[0], wh[1]);
+            B[0] = gather_exact<KT, L + 1>((const char *)pb + 8, 16, RX, wt[0], wh[1]);
+            E[2] = gather_exact<KT, KT>((const char *)p3, 8, RX, wt[0], wt[1]);
+            B[2] = gather_exact<L + 1, L + 1>((const char *)q3, 8, RX, wh[0], wh[1]);
+        } else {
+            int64_t v[6];
+            gather_pair_fx<L + 1, KT>(pa, RX, wh[0], wt[1], v[0], v[4]);  // E1, B2
+            gather_pair_fx<KT, L + 1>(pb, RX, wt[0], wh[1], v[1], v[3]);  // E2, B1
+            v[2] = gather_one_fx<KT, KT>(p3, RX, wt[0], wt[1]);
+            v[5] = gather_one_fx<L + 1, L + 1>(q3, RX, wh[0], wh[1]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            E[k] = field_value(v[k], st.emax[k]);
-            B[k] = field_value(v[3 + k], st.emax[3 + k]);
+            for (int k = 0; k < 3; ++k) {
+                E[k] = field_value(v[k], st.emax[k]);
+                B[k] = field_value(v[3 + k], st.emax[3 + k]);
+            }
         }
     }
 
@@ -406,10 +541,10 @@ template <int L, int KT, bool DET>
 __device__ void tile_fx(const RunDev &rd, char *smem, int64_t tile)
 {
     constexpr int W = fx_warps(L);
-    const StageFx st = stage_fx_carve(smem, (int)rd.reg_nodes);
+    const StageFx st = stage_fx_carve(smem, rd);
     const int tx = (int)(tile % rd.ntile[0]), ty = (int)(tile / rd.ntile[0]);
     const int x0 = tx * rd.tile[0], y0 = ty * rd.tile[1];
-    stage_fx_load<W>(rd, st, x0, y0);
+    stage_fx_load<L, W>(rd, st, x0, y0);
     const Hot2D h = make_hot2d(rd);
     __syncthreads();
     for (int s = 0; s < rd.nsp; ++s) {
