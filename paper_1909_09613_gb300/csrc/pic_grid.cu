@@ -345,9 +345,9 @@ __global__ void __launch_bounds__(kBlock) k_kinetic(const __grid_constant__ RunD
 // S0 the Esirkepov deposit starts from, evaluated in 62-bit fixed point (pic_fixed.cuh); in FP64
 // they bound the kernel (k_kinetic has the figures).  A block takes a share (blockIdx.y of
 // gridDim.y) of one tile's particles of species blockIdx.z and sums them in shared memory, kRhoEpoch
-// particles at a time: 64-bit words in units of 2^(k - 62) for at most 2^k particles, so no sum
-// overflows and each product is rounded at 2^(k - 63) <= 2^-51 of a weight of 1, where FP64 sums of
-// dense cells round at 2^-50.  A word is two 32-bit atomics, the low one's carry going to the high
+// particles at a time: 64-bit words in units of 2^(k - 62), k = b - 2 for fewer than 2^b particles, so
+// that no sum reaches 2^64 and each product is rounded at 2^(k - 63) <= 2^-53 of a weight of 1, the
+// rounding of an FP64 sum there.  A word is two 32-bit atomics, the low one's carry going to the high
 // one.  The window covers particles up to `drift` cells away from their tile; what lies outside, and
 // everything when no window fits (nodes = 0), goes to the global density one reduction per node,
 // which is what bounded the kernel when every particle did
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kBlock) k_kinetic(const __grid_constant__ RunD
 // share a cell, and their atomics would collide, while particles about a cell's occupancy apart
 // (at most 32) sit in neighbouring cells; in the slot-major order neighbours in the store already
 // do (sh = 0).
-constexpr int kRhoEpoch = 4096;
+constexpr int kRhoEpoch = 4095;
 
 struct RhoWin {
     int drift[3], pre[3], w[3];
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kBlock) k_rho(const __grid_constant__ RunDev r
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t e = a; e < b; e += kRhoEpoch) {  // block-uniform
         const int cnt = (int)min(b - e, (int64_t)kRhoEpoch);
-        const int k = 32 - __clz(cnt - 1);  // cnt <= 2^k (a count of 1: k = 0)
+        const int k = max(30 - __clz(cnt), 0);  // cnt < 2^(k + 2)
         for (int i = threadIdx.x; i < 2 * win.nodes; i += kBlock) words[i] = 0;
         __syncthreads();
         const int passes = (cnt + (32 << sh) - 1) / (32 << sh) << sh;
