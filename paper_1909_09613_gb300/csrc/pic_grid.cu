@@ -343,15 +343,19 @@ __global__ void __launch_bounds__(kBlock) k_kinetic(const __grid_constant__ RunD
 
 // rho = sum q w W_l / V_c at integer nodes: the l + 1 non-zero B-spline weights per axis, the same
 // S0 the Esirkepov deposit starts from, evaluated in 62-bit fixed point (pic_fixed.cuh); in FP64
-// they bound the kernel (k_kinetic has the figures).  A block takes a share (blockIdx.y of
-// gridDim.y) of one tile's particles of species blockIdx.z and sums them in shared memory, kRhoEpoch
-// particles at a time: 64-bit words in units of 2^(k - 62), k = b - 2 for fewer than 2^b particles, so
+// they bound the kernel (k_kinetic has the figures).  A block takes an equal share of the particles of
+// species blockIdx.y, whatever the tiles hold, with its ends moved to a tile's where one is near
+// (rho_edge), and sums every tile's part of it in shared memory, kRhoEpoch particles at a time: 64-bit words in units of 2^(k - 62), k = b - 2 for fewer than 2^b particles, so
 // that no sum reaches 2^64 and each product is rounded at 2^(k - 63) <= 2^-53 of a weight of 1, the
 // rounding of an FP64 sum there.  A word is two 32-bit atomics, the low one's carry going to the high
-// one.  The window covers particles up to `drift` cells away from their tile; what lies outside, and
-// everything when no window fits (nodes = 0), goes to the global density one reduction per node,
-// which is what bounded the kernel when every particle did
-// (pic_diag of 134M particles 10.6 -> 7.5 ms, FP32 form, and 11.7 -> 6.7 ms, FP64 form).
+// one.  The window covers particles up to `drift` cells away from their tile; what lies outside, tiles of
+// few particles, and everything when no window fits (nodes = 0), goes to the global density one
+// reduction per node, which is what bounded the kernel when every particle did
+// (pic_diag of 134M particles 10.6 -> 7.5 ms, FP32 form, and 11.7 -> 6.7 ms, FP64 form).  Equal
+// shares instead of equal parts of every tile cost an even plasma 3% (2048x1024 quadratic, 8 of a
+// species per cell: 2.11 -> 2.18 ms, the search for the ends) and spare a dense one the walk
+// of its few full tiles by a few blocks (all particles in 1% of the cells 3.2 -> 2.2 ms, in 0.1% 11.8
+// -> 2.2; FP32 form 6.8 -> 2.8 and 29.8 -> 2.9).
 // The lanes of a warp take particles 2^sh apart: in the cell-major order neighbours in the store
 // share a cell, and their atomics would collide, while particles about a cell's occupancy apart
 // (at most 32) sit in neighbouring cells; in the slot-major order neighbours in the store already
@@ -361,6 +365,7 @@ constexpr int kRhoEpoch = 4095;
 struct RhoWin {
     int drift[3], pre[3], w[3];
     int nodes;
+    int64_t least;  // particles of a tile from which the window pays
 };
 
 // *(hi, lo) += v
@@ -373,8 +378,9 @@ __device__ __forceinline__ void shared_add64(uint32_t *lo, uint32_t *hi, uint64_
 
 template <int L, int DIM>
 __device__ __forceinline__ void rho_particle(const RunDev &rd, const SpeciesDev &sp,
-                                             const RhoWin &win, const int *org, int64_t p, int k,
-                                             uint32_t *lo, uint32_t *hi, double qw, double *rho)
+                                             const RhoWin &win, bool window, const int *org,
+                                             int64_t p, int k, uint32_t *lo, uint32_t *hi, double qw,
+                                             double *rho)
 {
     int c[3] = {0, 0, 0};
     uint64_t f[DIM];
@@ -394,7 +400,7 @@ __device__ __forceinline__ void rho_particle(const RunDev &rd, const SpeciesDev 
     }
     Limbs w[DIM][L + 1];
     int b[DIM], at[DIM];
-    bool in = win.nodes > 0;
+    bool in = window;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         uint64_t psi, t[L + 1];
@@ -443,6 +449,34 @@ __device__ __forceinline__ void rho_particle(const RunDev &rd, const SpeciesDev 
     }
 }
 
+// The tile of store position p (start[0] = 0 <= p < start[nt]), found by a whole warp together.
+__device__ __forceinline__ int64_t tile_of(const int64_t *start, int64_t nt, int64_t p)
+{
+    const int lane = threadIdx.x & 31;
+    int64_t a = 0, b = nt;  // start[a] <= p < start[b]
+    while (b - a > 1) {
+        const int64_t step = (b - a + 31) / 32, at = a + (lane + 1) * step;
+        a += __popc(__ballot_sync(0xffffffffu, at < b && start[at] <= p)) * step;
+        b = min(b, a + step);
+    }
+    return a;
+}
+
+// First particle of block i of nb and its tile (-1: to be searched for): the equal share's, or a
+// tile's first where one lies within half a share of it, so that a plasma of even density is divided
+// into whole tiles.
+__device__ __forceinline__ longlong2 rho_edge(const int64_t *start, int64_t nt, int64_t n, int64_t i,
+                                              int64_t nb)
+{
+    const int64_t p = n * i / nb, near = n / (2 * nb);
+    if (p >= n) return make_longlong2(n, -1);
+    const int64_t t = tile_of(start, nt, p), below = p - start[t], above = start[t + 1] - p;
+    if (below <= near && below <= above) return make_longlong2(p - below, t);
+    if (above > near) return make_longlong2(p, t);
+    // (tiles may be empty: the next particle's is not always t + 1)
+    return make_longlong2(p + above, start[min(t + 2, nt)] > p + above ? t + 1 : -1);
+}
+
 template <int L, int DIM>
 __global__ void __launch_bounds__(kBlock) k_rho(const __grid_constant__ RunDev rd,
                                                 const __grid_constant__ RhoWin win, int sh,
@@ -450,42 +484,82 @@ __global__ void __launch_bounds__(kBlock) k_rho(const __grid_constant__ RunDev r
 {
     extern __shared__ uint32_t words[];  // low words, then high words
     uint32_t *lo = words, *hi = words + win.nodes;
-    const SpeciesDev &sp = rd.sp[blockIdx.z];
-    const int64_t t = blockIdx.x, a0 = sp.tile_start[t], len = sp.tile_start[t + 1] - a0;
-    const int64_t a = a0 + len * blockIdx.y / gridDim.y, b = a0 + len * (blockIdx.y + 1) / gridDim.y;
-    int org[3];
-    org[0] = (int)(t % rd.ntile[0]) * rd.tile[0];
-    org[1] = (int)(t / rd.ntile[0] % rd.ntile[1]) * rd.tile[1];
-    org[2] = (int)(t / rd.ntile[0] / rd.ntile[1]) * rd.tile[2];
+    const SpeciesDev &sp = rd.sp[blockIdx.y];
+    const int64_t *start = sp.tile_start;
+    const int64_t n = sp.n, nt = rd.ntiles, nb = gridDim.x, none = win.nodes == 0;
+    if (n == 0) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ longlong2 edge[2];
+    int64_t first = n * blockIdx.x / nb, last = n * (blockIdx.x + 1) / nb, tile = 0;
+    if (!none) {
+        if (warp < 2) {  // a search each, side by side
+            const longlong2 e = rho_edge(start, nt, n, blockIdx.x + warp, nb);
+            if (lane == 0) edge[warp] = e;
+        }
+        __syncthreads();
+        first = edge[0].x;
+        tile = edge[0].y;
+        last = edge[1].x;
+    }
     const double vc = rd.dx[0] * rd.dx[1] * (DIM == 3 ? rd.dx[2] : 1.0);
     const double qw = sp.q * sp.w / vc;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t e = a; e < b; e += kRhoEpoch) {  // block-uniform
-        const int cnt = (int)min(b - e, (int64_t)kRhoEpoch);
-        const int k = max(30 - __clz(cnt), 0);  // cnt < 2^(k + 2)
-        for (int i = threadIdx.x; i < 2 * win.nodes; i += kBlock) words[i] = 0;
-        __syncthreads();
-        const int passes = (cnt + (32 << sh) - 1) / (32 << sh) << sh;
-#pragma unroll 1
-        for (int i = warp; i < passes; i += kBlock / 32) {
-            const int q = ((i >> sh) << (5 + sh)) + (lane << sh) + (i & ((1 << sh) - 1));
-            if (q < cnt) rho_particle<L, DIM>(rd, sp, win, org, e + q, k, lo, hi, qw, rho);
-        }
-        __syncthreads();
-        const double unit = __hiloint2double((1023 + k - 62) << 20, 0);
-        const int rows = win.nodes / max(win.w[0], 1);
-        for (int r = warp; r < rows; r += kBlock / 32) {
-            const int ry = r % win.w[1], rz = r / win.w[1];
-            const int gy = wrap_near(org[1] - win.pre[1] + ry, rd.n[1]);
-            const int gz = DIM == 3 ? wrap_near(org[2] - win.pre[2] + rz, rd.n[2]) : 0;
-            double *row = rho + gidx(rd, 0, gy, gz);
-            for (int i = lane; i < win.w[0]; i += 32) {
-                const int n = r * win.w[0] + i;
-                const uint64_t v = (uint64_t)hi[n] << 32 | lo[n];
-                if (v) atomicAdd(row + wrap_near(org[0] - win.pre[0] + i, rd.n[0]), (double)v * unit * qw);
+    for (int64_t p = first; p < last;) {  // block-uniform
+        // what is summed together: the part of p's tile, or, with no window, all up to the next part
+        // that takes one
+        int64_t end = last;
+        bool window = false;
+        int org[3] = {0, 0, 0};
+        if (!none) {
+            int64_t t = p > first || tile < 0 ? tile_of(start, nt, p) : tile;
+            org[0] = (int)(t % rd.ntile[0]) * rd.tile[0];
+            org[1] = (int)(t / rd.ntile[0] % rd.ntile[1]) * rd.tile[1];
+            org[2] = (int)(t / rd.ntile[0] / rd.ntile[1]) * rd.tile[2];
+            end = max(min(last, start[t + 1]), p + 1);  // (start[t] <= p < start[t + 1])
+            window = end - p >= win.least;
+            while (!window && end < last) {  // 32 tiles at a time, the warp's lanes one each
+                const int64_t u = t + 1 + lane;
+                const int64_t s = u < nt ? min(start[u], last) : last;
+                const unsigned stop = __ballot_sync(
+                    0xffffffffu, s >= last || min(start[u + 1], last) - s >= win.least);
+                if (stop) {
+                    end = max(end, __shfl_sync(0xffffffffu, s, __ffs(stop) - 1));
+                    break;
+                }
+                t += 32;
             }
         }
-        __syncthreads();
+        const int64_t step = window ? kRhoEpoch : (int64_t)1 << 20;
+        for (; p < end; p += step) {
+            const int cnt = (int)min(end - p, step);
+            const int k = max(30 - __clz(cnt), 0);  // cnt < 2^(k + 2)
+            if (window) {
+                for (int i = threadIdx.x; i < 2 * win.nodes; i += kBlock) words[i] = 0;
+                __syncthreads();
+            }
+            const int passes = (cnt + (32 << sh) - 1) / (32 << sh) << sh;
+#pragma unroll 1
+            for (int i = warp; i < passes; i += kBlock / 32) {
+                const int q = ((i >> sh) << (5 + sh)) + (lane << sh) + (i & ((1 << sh) - 1));
+                if (q < cnt) rho_particle<L, DIM>(rd, sp, win, window, org, p + q, k, lo, hi, qw, rho);
+            }
+            if (!window) continue;
+            __syncthreads();
+            const double unit = __hiloint2double((1023 + k - 62) << 20, 0);
+            const int rows = win.nodes / win.w[0];
+            for (int r = warp; r < rows; r += kBlock / 32) {
+                const int ry = r % win.w[1], rz = r / win.w[1];
+                const int gy = wrap_near(org[1] - win.pre[1] + ry, rd.n[1]);
+                const int gz = DIM == 3 ? wrap_near(org[2] - win.pre[2] + rz, rd.n[2]) : 0;
+                double *row = rho + gidx(rd, 0, gy, gz);
+                for (int i = lane; i < win.w[0]; i += 32) {
+                    const int m = r * win.w[0] + i;
+                    const uint64_t v = (uint64_t)hi[m] << 32 | lo[m];
+                    if (v) atomicAdd(row + wrap_near(org[0] - win.pre[0] + i, rd.n[0]), (double)v * unit * qw);
+                }
+            }
+            __syncthreads();
+        }
+        p = end;
     }
 }
 
@@ -666,16 +740,19 @@ static cudaError_t launch_rho(const RunDev &rd, double *rho, cudaStream_t st)
     int sh = 0;
     while (!rd.slot_major && sh < 5 && (rd.ncell << (sh + 1)) <= n) ++sh;
     RhoWin win = rho_window(rd);
-    // zeroing and adding the window costs as much as what it saves below about eight
-    // contributions per node (FP64 96x40x36 quadratic, 4 of a species per cell: 4.8 per node, pic_diag
-    // 263 us without a window, 298 with; FP32 256x64x64 alike: 10.4 per node, 1120 and 1057)
-    double sums = (double)n / rd.ntiles;
-    for (int a = 0; a < rd.dim; ++a) sums *= rd.l + 1;
-    if (sums < 8.0 * win.nodes) win.nodes = 0;
-    // parts of a tile: enough blocks for a grid of few tiles, each of a thousand particles or more
+    // zeroing and adding the window costs as much as what it saves below about five to seven
+    // contributions per node (pic_diag without it / with it, us: FP64 96x40x36 quadratic 4.8 per node
+    // 238 / 235, 7.2 321 / 282, 9.6 406 / 333; 512x256 cubic 7.0 96 / 96, 14 120 / 109; FP32
+    // 128x64x64 quadratic 5.2 402 / 418, 10.4 746 / 591): the line lies at eight for the average
+    // tile, and at four for a single one of a run that takes windows
+    double per = 1.0;
+    for (int a = 0; a < rd.dim; ++a) per *= rd.l + 1;
+    if ((double)n / rd.ntiles * per < 8.0 * win.nodes) win.nodes = 0;
+    win.least = (int64_t)(4.0 * win.nodes / per);
+    // enough blocks for a grid of few tiles, each of a thousand particles or more
     const int64_t want = (2048 + rd.ntiles - 1) / rd.ntiles, most = n / rd.ntiles / 1024;
     const int64_t parts = want < most ? want : most;
-    const dim3 g((unsigned)rd.ntiles, (unsigned)(parts > 1 ? parts : 1), rd.nsp);
+    const dim3 g((unsigned)(rd.ntiles * (parts > 1 ? parts : 1)), rd.nsp);
     const bool d3 = rd.dim == 3;
     auto k = rd.l == 1 ? (d3 ? k_rho<1, 3> : k_rho<1, 2>)
              : rd.l == 2 ? (d3 ? k_rho<2, 3> : k_rho<2, 2>)
