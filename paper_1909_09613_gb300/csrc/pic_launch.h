@@ -50,10 +50,14 @@ constexpr int64_t kEvenMin = 1024;
 // (EvenSplit).  Whole tiles or whole parts of them left slots empty in a grid of few waves: 256
 // tiles, or 64 tiles in 4 parts, are 256 CTAs on 304 slots.  A share that crosses a tile border
 // stages twice and still wins (particle kernel, us, 512x256 at 32 per cell: quadratic 212 -> 193,
-// cubic 229 -> 200; 256x128 quartic at 64 per cell 168 -> 162).
+// cubic 229 -> 200; 256x128 quartic at 64 per cell 168 -> 162).  Where the lines lie (whole parts /
+// even shares, us, 256x128): 431 particles of a species per CTA quadratic 45.7 / 47.6, 647 cubic 61.0 /
+// 63.2, 862 cubic 69.5 / 66.9, 1293 cubic 81.1 / 78.8.  A deterministic run's CTAs are counted for the
+// slots of a GB300 whatever the device: its warps add their lanes' FP32 currents before the fixed-point
+// word, so which 32 particles meet must not depend on the device.
 inline unsigned tile_ctas(const RunDev &rd)
 {
-    const int64_t slots = tile_slots(), per_tile = tile_load(rd), nt = rd.ntiles;
+    const int64_t slots = rd.det ? 304 : tile_slots(), per_tile = tile_load(rd), nt = rd.ntiles;
     // whole parts per tile, as many as fill the slots once, down to one warp of each species
     int64_t parts = slots / nt;
     const int64_t most = (per_tile + 31) / 32;
