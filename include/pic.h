@@ -127,7 +127,9 @@ int pic_create(const int32_t grid[3], const double dx[3], double dt, int spline_
 int pic_footprint(const pic_ctx *ctx, size_t *bytes);
 
 /* Hand the context a device buffer of at least pic_footprint bytes (e.g. a torch tensor's
- * storage).  The caller keeps it alive until pic_destroy.  The fields are zeroed.            */
+ * storage).  The caller keeps it alive until pic_destroy.  The fields are zeroed.  The first call
+ * of a process page-locks 320 kB of the library's own memory, which small reads pass through and
+ * which stays locked.                                                                        */
 int pic_bind_memory(pic_ctx *ctx, void *dev_ptr, size_t bytes);
 
 /* Alternative to pic_bind_memory: the library allocates (cudaMalloc) and frees the buffer. */

@@ -73,8 +73,11 @@ namespace {
 // pageable memory costs 7 to 14 us more than one into page-locked memory: 16 kB with its error word
 // 26 us, through the stage 13; 252 kB 31 and 26; from there the stage's second copy costs more (1 MB
 // 38 and 75).  A 64x32 run: nine fields 294 -> 222 us, two species' particles 185 -> 98 us.  One
-// block serves every context (one that finds no slot, or the stage in use by another thread, copies
-// directly) and is freed with the last.
+// block of 320 kB serves every context (one that finds no slot, or the stage in use by another thread,
+// copies directly).  It is the library's own static memory, page-locked when the first run is bound
+// and left so: locking and releasing it wait for the whole device, and a program that makes and
+// drops one run at a time would do both for every run.  (A device reset releases it; the next run
+// bound locks it again.)
 class Pinned {
   public:
     static constexpr size_t kSlot = 64, kStage = 256 * 1024;
@@ -82,13 +85,9 @@ class Pinned {
     char *take()
     {
         std::lock_guard<std::mutex> lock(mu_);
-        if (!block_) {
-            void *p = nullptr;
-            if (cudaHostAlloc(&p, kSlots * kSlot + kStage, cudaHostAllocPortable) != cudaSuccess) {
-                cudaGetLastError();
-                return nullptr;
-            }
-            block_ = (char *)p;
+        if (live_ == 0 && !locked() && cudaHostRegister(block_, sizeof(block_), cudaHostRegisterPortable) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
         }
         for (int i = 0; i < kSlots; ++i)
             if (!used_[i]) {
@@ -103,12 +102,9 @@ class Pinned {
         if (!slot) return;
         std::lock_guard<std::mutex> lock(mu_);
         used_[(slot - block_) / kSlot] = false;
-        if (--live_ == 0) {
-            cudaFreeHost(block_);
-            block_ = nullptr;
-        }
+        --live_;
     }
-    // the stage, for a caller that holds a slot (so the block stays) and lock for its whole use
+    // the stage, for a caller that holds a slot (so the block is locked) and lock for its whole use
     char *stage(std::unique_lock<std::mutex> &lock, const char *slot, size_t bytes)
     {
         if (!slot || bytes > kStage) return nullptr;
@@ -118,10 +114,21 @@ class Pinned {
 
   private:
     static constexpr int kSlots = 1024;
+
+    bool locked()
+    {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, block_) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return a.type == cudaMemoryTypeHost;
+    }
+
     std::mutex mu_, stage_mu_;
-    char *block_ = nullptr;
     int live_ = 0;
     bool used_[kSlots] = {};
+    alignas(4096) char block_[kSlots * kSlot + kStage];
 };
 Pinned g_pinned;
 constexpr int kErrAt = 48;  // the error word's place in a slot, after six doubles of diagnostics
