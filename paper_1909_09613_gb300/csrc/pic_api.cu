@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 
@@ -104,10 +105,19 @@ class Pinned {
         used_[(slot - block_) / kSlot] = false;
         --live_;
     }
-    // the stage, for a caller that holds a slot (so the block is locked) and lock for its whole use
-    char *stage(std::unique_lock<std::mutex> &lock, const char *slot, size_t bytes)
+    // the stage, for a caller that holds a slot (so the block is locked) and lock for its whole use; not
+    // for destinations in device memory, which a direct copy reaches and the host does not
+    char *stage(std::unique_lock<std::mutex> &lock, const char *slot, size_t bytes,
+                std::initializer_list<const void *> to)
     {
         if (!slot || bytes > kStage) return nullptr;
+        for (const void *p : to) {
+            cudaPointerAttributes a;
+            if (p && (cudaPointerGetAttributes(&a, p) != cudaSuccess || a.type == cudaMemoryTypeDevice)) {
+                cudaGetLastError();
+                return nullptr;
+            }
+        }
         lock = std::unique_lock<std::mutex>(stage_mu_, std::try_to_lock);
         return lock.owns_lock() ? block_ + kSlots * kSlot : nullptr;
     }
@@ -930,7 +940,7 @@ int pic_read_fields(pic_ctx *c, int comp, double *host, size_t count)
     if (count != (size_t)c->rd.ncell) return PIC_EINVAL;
     const size_t bytes = count * sizeof(double);
     std::unique_lock<std::mutex> lock;
-    char *stage = g_pinned.stage(lock, c->pinned, bytes);
+    char *stage = g_pinned.stage(lock, c->pinned, bytes, {host});
     if (cudaMemcpyAsync(stage ? (void *)stage : host, c->rd.F[comp], bytes, cudaMemcpyDeviceToHost,
                         c->stream) != cudaSuccess)
         return PIC_ECUDA;
@@ -952,7 +962,7 @@ int pic_read_particles(pic_ctx *c, int species, double *x, double *u, int64_t *c
     // few particles: all arrays in one copy through the page-locked stage
     const size_t all = (size_t)np * ((d + 3) * sizeof(double) + sizeof(int64_t));
     std::unique_lock<std::mutex> lock;
-    if (char *stage = np <= kChunk ? g_pinned.stage(lock, c->pinned, all) : nullptr) {
+    if (char *stage = np <= kChunk ? g_pinned.stage(lock, c->pinned, all, {x, u, cell}) : nullptr) {
         double *sx = (double *)c->staging, *su = sx + (size_t)d * np;
         if (launch_unpack(c->rd, species, sx, su, (int64_t *)(su + (size_t)3 * np), np, 0, c->stream)
             != cudaSuccess)
