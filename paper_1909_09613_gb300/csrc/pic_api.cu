@@ -156,15 +156,6 @@ size_t staging_size(const RunDev &rd, int64_t capmax)
 
 int pos_bytes(const pic_ctx *c) { return c->rd.prec == PIC_FP32_MIXED ? 4 : 8; }
 
-// FP64 2D, l <= 3: bytes the footprint keeps per species beyond what the run uses (room for
-// 2 (l + 1) FP64 values per particle of capacity, which the particle pass once cached), so that
-// buffers and admission budgets sized by it stay what they were.
-size_t reserved_bytes(const pic_ctx *c, int s)
-{
-    if (c->rd.prec != PIC_FP64 || c->rd.dim != 2 || c->rd.l > 3) return 0;
-    return (size_t)c->cap[s] * 2 * (c->rd.l + 1) * sizeof(double);
-}
-
 int particle_bytes(const pic_ctx *c)
 {
     const int d = c->rd.dim;
@@ -629,6 +620,38 @@ static bool uses_j32(const RunDev &rd)
     return rd.dim == 3 && rd.prec == PIC_FP32_MIXED && !rd.det;
 }
 
+// Where the staging buffer's bytes go besides loads and read-backs, which use it in stream order and
+// never across a sort or within a call of pic_step: the sort scratch of the further species, then
+// (FP64 form) the y and z components of the copy of B that the gather of a call's steps reads -- each
+// where it fits.  (Its x component lies in the charge density, which nothing holds between calls.)
+struct StagingUse {
+    size_t sort, b;  // bytes; 0: not in the staging buffer
+};
+
+static StagingUse staging_use(const RunDev &rd, int64_t capmax)
+{
+    const size_t room = staging_size(rd, capmax);
+    const int64_t keys = rd.ntiles * rd.tile[0] * rd.tile[1] * rd.tile[2];
+    StagingUse u;
+    u.sort = align_up((size_t)(rd.nsp - 1) * sort_set_bytes(keys, rd.ntiles, capmax), 256);
+    if (u.sort > room) u.sort = 0;
+    u.b = rd.prec == PIC_FP64 ? 2 * align_up(rd.ncell * sizeof(double), 256) : 0;
+    if (u.sort + u.b > room) u.b = 0;
+    return u;
+}
+
+// What the scratch of a run takes at least in its footprint.  The cubic FP64 2D form's is counted for
+// 64 B per particle of capacity, which its footprint has always had beside the particle stores (for
+// weights that are no longer cached) and buffers and estimates are sized by: the scratch lies in it.
+static size_t least_scratch(const pic_ctx *c)
+{
+    const RunDev &rd = c->rd;
+    size_t b = 0;
+    if (rd.prec == PIC_FP64 && rd.dim == 2 && rd.l == 3)
+        for (int s = 0; s < rd.nsp; ++s) b += align_up((size_t)c->cap[s] * 64, 256);
+    return b;
+}
+
 int pic_footprint(const pic_ctx *c, size_t *bytes)
 {
     if (!c || !bytes) return PIC_EINVAL;
@@ -638,28 +661,24 @@ int pic_footprint(const pic_ctx *c, size_t *bytes)
     b += 9 * align_up(rd.ncell * sizeof(double), A);                           // F
     if (rd.prec == PIC_FP32_MIXED) b += 6 * align_up(rd.ncell * sizeof(float), A);  // Fs
     const int pb = particle_bytes(c);
-    int64_t capmax = 0, captot = 0;
-    for (int s = 0; s < rd.nsp; ++s) {
-        capmax = std::max(capmax, c->cap[s]);
-        captot += c->cap[s];
-    }
+    int64_t capmax = 0;
+    for (int s = 0; s < rd.nsp; ++s) capmax = std::max(capmax, c->cap[s]);
     const int TC = rd.tile[0] * rd.tile[1] * rd.tile[2];
-    for (int s = 0; s < rd.nsp; ++s) b += align_up((size_t)c->cap[s] * pb + 7 * A, A);  // current stores
-    for (int s = 0; s < rd.nsp; ++s) b += align_up((rd.ntiles + 1) * sizeof(int64_t), A);           // tile_start
-    for (int s = 0; s < rd.nsp; ++s) b += align_up(reserved_bytes(c, s), A);
-    // sort targets and sort scratch
-    for (int s = 0; s < rd.nsp; ++s) b += align_up((size_t)c->cap[s] * pb + 7 * A, A);
-    b += 2 * align_up(rd.ntiles * TC * sizeof(int32_t), A);
-    b += 4 * align_up((size_t)capmax * sizeof(int32_t), A);
-    b += align_up((rd.ntiles + 1) * sizeof(int64_t), A);
-    b += staging_size(rd, capmax);                // host<->device staging (chunked)
-    b += 3 * align_up(rd.ncell * sizeof(double), A);  // rho, rho_prev, gref
-    if (rd.det && rd.prec == PIC_FP64) b += 3 * align_up(rd.ncell * sizeof(double), A);  // jlo
-    if (uses_j32(rd)) b += align_up(3 * rd.jp_nodes * sizeof(float), A);                // J32
-    if (rd.prec == PIC_FP64) b += 3 * align_up(rd.ncell * sizeof(double), A);           // Bg
+    // current stores, sort targets, tile_start
+    for (int s = 0; s < rd.nsp; ++s) b += 2 * align_up((size_t)c->cap[s] * pb + 7 * A, A);
+    for (int s = 0; s < rd.nsp; ++s) b += align_up((rd.ntiles + 1) * sizeof(int64_t), A);
+    size_t w = 0;
+    w += 2 * align_up(rd.ntiles * TC * sizeof(int32_t), A);  // sort scratch
+    w += 4 * align_up((size_t)capmax * sizeof(int32_t), A);
+    w += align_up((rd.ntiles + 1) * sizeof(int64_t), A);
+    w += staging_size(rd, capmax);                // host<->device staging (chunked)
+    w += 3 * align_up(rd.ncell * sizeof(double), A);  // rho, rho_prev, gref
+    if (rd.det && rd.prec == PIC_FP64) w += 3 * align_up(rd.ncell * sizeof(double), A);  // jlo
+    if (uses_j32(rd)) w += align_up(3 * rd.jp_nodes * sizeof(float), A);                // J32
+    if (rd.prec == PIC_FP64 && !staging_use(rd, capmax).b) w += 2 * align_up(rd.ncell * sizeof(double), A);  // Bg
+    b += std::max(w, least_scratch(c));
     b += 2 * A;                                   // diag out, err
     b += A;                                       // base alignment slack
-    (void)captot;
     *bytes = b;
     return PIC_OK;
 }
@@ -709,13 +728,9 @@ int pic_bind_memory(pic_ctx *c, void *dev, size_t bytes)
     c->sc.tile_count = (int64_t *)take((rd.ntiles + 1) * sizeof(int64_t));
     c->staging_bytes = staging_size(rd, capmax);
     c->staging = take(c->staging_bytes);
-    // the further species' sort scratch lies in the staging buffer, where it fits (up to kChunk
-    // particles of a species): loads and read-backs use it in stream order, never across a sort
-    rd.sc_more = nullptr;
+    const StagingUse use = staging_use(rd, capmax);
+    rd.sc_more = use.sort ? c->staging : nullptr;
     rd.sc_cap = capmax;
-    if (rd.nsp > 1
-        && (rd.nsp - 1) * sort_set_bytes(rd.ntiles * TC, rd.ntiles, capmax) <= (int64_t)c->staging_bytes)
-        rd.sc_more = c->staging;
     c->rho = (double *)take(rd.ncell * sizeof(double));
     c->rho_prev = (double *)take(rd.ncell * sizeof(double));
     c->gref = (double *)take(rd.ncell * sizeof(double));
@@ -730,8 +745,14 @@ int pic_bind_memory(pic_ctx *c, void *dev, size_t bytes)
         float *j = (float *)take(3 * rd.jp_nodes * sizeof(float));
         for (int a = 0; a < 3; ++a) rd.J32[a] = j + a * rd.jp_nodes;
     }
-    for (int a = 0; a < 3; ++a)
-        rd.Bg[a] = rd.prec == PIC_FP64 ? (double *)take(rd.ncell * sizeof(double)) : nullptr;
+    for (int a = 0; a < 3; ++a) rd.Bg[a] = nullptr;
+    if (rd.prec == PIC_FP64) {
+        const size_t n = align_up(rd.ncell * sizeof(double), A);
+        char *at = use.b ? c->staging + use.sort : take(2 * n);
+        rd.Bg[0] = c->rho;
+        rd.Bg[1] = (double *)at;
+        rd.Bg[2] = (double *)(at + n);
+    }
     c->rho_prev_valid = false;
     c->gref_valid = false;
     c->diag_out = (double *)take(8 * sizeof(double));
