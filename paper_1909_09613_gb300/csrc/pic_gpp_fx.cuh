@@ -11,10 +11,10 @@
 // evaluation read from a per-particle cache (128 B per particle and step), are evaluated.
 //
 // The gather's signed, rounded sums and the search for tiles whose fields one scale does not resolve
-// cost 6% of it (512x256, cubic, 32 of a species per cell, 8.4 M particles: 3.11 -> 3.32 ms; 64x32 at
-// 8: 37.6 -> 41.3 us, most of it the search) against biased sums of truncated products, which gave a
-// particle a one-signed field of 2^-54 of the tile's largest where its own was zero, and a node below
-// 2^-6 of the largest fewer bits than FP64.
+// cost 2 to 9% of it (cubic, 512x256 at 32 and 8 of a species per cell 3.11 -> 3.18 and 0.848 -> 0.905 ms,
+// 64x32 at 8 37.6 -> 41.1 us, most of it the search) against biased sums of truncated products, which
+// gave a particle a one-signed field of 2^-54 of the tile's largest where its own was zero, and a node
+// below 2^-6 of the largest fewer bits than FP64.
 #pragma once
 #include "pic_fixed.cuh"
 #include "pic_gpp_kernels.cuh"
@@ -36,8 +36,12 @@ struct StageFx {
 };
 
 // Warps of a block, two blocks per SM.  Quartic splines spill at the 128 registers of 16 warps per
-// SM as they do at the 96 of 20, and the extra warps hide more of the wait (255x130 at 16 per cell
-// 338 -> 316 us); cubic ones do not spill and lose (134M particles 40.7 -> 42.5 ms).
+// SM as they do at the 96 of 20, and the extra warps hide more of the wait (8 / 10 warps, us: 255x130
+// at 2, 8 and 32 of a species per cell 105 / 101, 386 / 348, 1334 / 1252; 512x256 at 4 and 16 675 / 657,
+// 2523 / 2445; 1024x512 at 16 9580 / 9602; the other way 128x64 at 8 90 / 97, 512x256 at 32 4766 /
+// 4952).  Deterministic runs spill with ten warps only and are faster with them all the same (255x130
+// at 8 734 / 715, 512x256 at 32 9594 / 9499).  Cubic splines do not spill and lose (134M particles
+// 40.7 -> 42.5 ms).
 __host__ __device__ constexpr int fx_warps(int l) { return l == 4 ? 10 : 8; }
 
 constexpr int kFxHead = 2 * sizeof(TTable) + 32;  // tables, exponents and the exact flag

@@ -98,3 +98,17 @@ def test_fixed_point_weights_equal_the_fp64_ones(host, l, scheme, dtt):
         a[12 + base[i]: 12 + base[i] + k] = w[i]
         b[12 + b0: 12 + b0 + len(w0)] = w0
         assert np.max(np.abs(a - b)) <= 4e-15, (d, dtt, base[i], b0)
+
+
+@pytest.mark.parametrize("l", [1, 2, 3, 4])
+@pytest.mark.parametrize("dtt", [0.25, 0.6, 1e-3, 1e-6, 1e-9])
+def test_fixed_point_weights_sum_to_one(host, l, dtt):
+    """In units of 2^-62, but where the others leave nothing for the middle weight, which is not
+    negative (a few units of 2^-59 each; the table's own rounding of 2^-64 / dtt in the others)."""
+    f = np.random.default_rng(l).integers(0, 2 ** 64, 2000, dtype=np.uint64)
+    base, w = np.zeros(len(f), dtype=np.int32), np.zeros(6 * len(f), dtype=np.uint64)
+    k = host.weights62(l, pic.PIC_SCHEME_WT, dtt, f.ctypes.data, len(f), base.ctypes.data, w.ctypes.data)
+    w = w[: k * len(f)].reshape(len(f), k)
+    left = w.sum(axis=1).astype(np.int64) - 2 ** 62
+    assert np.all((left == 0) | ((w[:, k // 2] == 0) & (left > 0) & (left < 8 * 30 + 2 / dtt)))
+    assert l == 1 or np.all(left == 0)
