@@ -19,6 +19,7 @@ cudaError_t launch_gpp_f64(const RunDev &rd, int kt, cudaStream_t st);
 size_t gpp_smem_bytes_f32(const RunDev &rd);
 size_t gpp_batch_smem_bytes_f32(const RunDev &rd);
 size_t gpp_smem_bytes_f64(const RunDev &rd);
+size_t gpp_launch_smem_bytes_f64(const RunDev &rd);
 }  // namespace pic
 
 struct pic_ctx {
@@ -1050,7 +1051,8 @@ int pic_smem_info(const pic_ctx *c, size_t *own_bytes, size_t *batched_bytes,
                   size_t *two_per_sm_bytes)
 {
     if (!c) return PIC_EINVAL;
-    if (own_bytes) *own_bytes = c->smem;
+    if (own_bytes)
+        *own_bytes = c->rd.prec == PIC_FP64 && c->rd.dim == 2 ? gpp_launch_smem_bytes_f64(c->rd) : c->smem;
     if (batched_bytes)
         *batched_bytes = c->rd.prec == PIC_FP32_MIXED ? gpp_batch_smem_bytes_f32(c->rd) : 0;
     if (two_per_sm_bytes) {

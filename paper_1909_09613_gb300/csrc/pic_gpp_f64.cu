@@ -39,6 +39,9 @@ cudaError_t launch_gpp_f64(const RunDev &rd, int kt, cudaStream_t st)
     }
 }
 
+// What a 2D launch takes, and what it must have.
+size_t gpp_launch_smem_bytes_f64(const RunDev &rd) { return stage_fx_launch_bytes(rd); }
+
 size_t gpp_smem_bytes_f64(const RunDev &rd)
 {
     return rd.dim == 2 ? stage_fx_bytes(rd.reg_nodes) : 0;
