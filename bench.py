@@ -790,15 +790,25 @@ def main():
     except Exception:
         pass
     ach = alg_bytes / gpp_avg_s / 1e9
-    roofline = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": ach / peaks["hbm_gbs"], "traffic": traffic64,
-                "peak_source": "%s hbm_gbs" % peak_kind,
-                "note": "bound on chip: the weights, gather and current products run on the "
-                        "integer units in 62-bit fixed point, the push on the FP64 pipe"}
-    instr = c64.get("fp64_pipe_instr_per_particle")
-    if instr and fp64_peak:  # the FP64 pipe completes peak / 2 instructions per second
-        roofline["fp64_pipe_frac"] = res["n"] * instr / gpp_avg_s / (fp64_peak * 1e12 / 2.0)
-        roofline["warp_instr_per_particle"] = c64.get("warp_instr_per_particle")
+    hbm = {"achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
+           "peak_source": "%s hbm_gbs" % peak_kind}
+    warp = c64.get("warp_instr_per_particle")
+    mhz = (res["clocks"] or {}).get("sm_mhz")
+    if warp and mhz:
+        # bound on chip: weights, gather and current products run on the integer units in 62-bit
+        # fixed point, the push on the FP64 pipe; what all of them share is the issue slots
+        rate, peak = res["n"] * warp / gpp_avg_s / 1e9, sms * SCHEDULERS_PER_SM * mhz * 1e-3
+        roofline = {"bound": "issue", "achieved": rate, "peak": peak, "unit": "G warp instructions/s",
+                    "frac": rate / peak, "traffic": traffic64, "warp_instr_per_particle": warp,
+                    "peak_source": "%d SMs x %d issue slots x the SM clock under load"
+                                   % (sms, SCHEDULERS_PER_SM),
+                    "hbm_view": hbm}
+        instr = c64.get("fp64_pipe_instr_per_particle")
+        if instr and fp64_peak:  # the FP64 pipe completes peak / 2 instructions per second
+            roofline["fp64_pipe_frac"] = res["n"] * instr / gpp_avg_s / (fp64_peak * 1e12 / 2.0)
+    else:
+        roofline = dict(hbm, bound="hbm", traffic=traffic64,
+                        note="no instruction counts recorded for these kernel sources")
     roofline["kernel"] = "k_gpp2d<3,4> (double): fused gather+push+move+deposit"
     roofline["kernel_ms"] = gpp_avg_s * 1e3
     roofline["algorithmic_bytes"] = alg_bytes
