@@ -7,7 +7,7 @@
 // interpolation stencils and the drift since the last sort) in shared memory, walks the tile's
 // particles (contiguous in the sorted store), gathers, pushes and moves them.  The FP32 form sums
 // its lanes' currents through shared memory into a J tile that is added to the global FP64
-// current with one atomic per tile node and component; the FP64 form adds every contribution to
+// current with one atomic per tile node, component and species; the FP64 form adds every contribution to
 // the global current as an L2 reduction.  In 3D
 // the FP32 form stages its tile's fields in shared memory too (the FP64 form reads them through
 // L1), and every current contribution goes straight to a global reduction (FP32 form: into an

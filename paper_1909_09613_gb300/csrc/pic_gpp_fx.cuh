@@ -2,11 +2,11 @@
 // 62-bit fixed point (pic_fixed.cuh), Boris push and move in FP64.
 //
 // What bounds it: an FP64 evaluation is bound by the FP64 pipe (2 operations per clock and SM, 410
-// of them per particle for cubic splines).  In fixed point 81 stay there (Boris, move, the
+// of them per particle for cubic splines).  In fixed point 78 stay there (Boris, move, the
 // interpolated fields' conversion) and the rest goes to the integer units; the pipes are then
 // about equally loaded (FP64 39%, wide multiplier 54%, ALU 43% of their cycles, 52% of the issue
 // slots) and the warps wait on fixed-latency dependencies.  512x256, cubic, 64 per cell: 7.39 ->
-// 2.70 ms per pass over 8.4 M particles; 255x130, quartic, 16 per cell: 0.72 -> 0.34 ms.  Three
+// 2.70 ms per pass over 8.4 M particles (now 2.76); 255x130, quartic, 16 per cell: 0.72 -> 0.34 ms.  Three
 // CTAs per SM at 80 registers spill (2.90 ms).  The old-position weights, which the FP64
 // evaluation read from a per-particle cache (128 B per particle and step), are evaluated.
 //
