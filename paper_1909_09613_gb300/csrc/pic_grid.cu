@@ -576,7 +576,7 @@ RhoWin rho_window(const RunDev &rd)
         w.w[a] = on ? rd.tile[a] + w.drift[a] + w.pre[a] + rd.l - (rd.l - 1) / 2 : 1;
         nodes *= w.w[a];
     }
-    w.nodes = nodes * 8 <= 48 * 1024 ? (int)nodes : 0;
+    w.nodes = nodes * 8 <= 47 * 1024 ? (int)nodes : 0;  // (48 KB, some of it the kernel's own)
     return w;
 }
 

@@ -73,3 +73,22 @@ def test_uneven_plasma_matches_oracle(grid, l, counts, share, prec):
     assert abs(got - abs(left)) <= 1e-10 * size
     run.close()
     orc.close()
+
+
+def test_largest_window():
+    """Tiles of 1 x 17 x 25 cells and their reach are 8 x 24 x 32 = 6,144 nodes, 48 KB of words: the most
+    shared memory a launch takes unasked, of which the kernel needs a little besides."""
+    grid, n = (4, 17, 25), 40000
+    rng = np.random.default_rng(4)
+    run = pic.Run(grid, (1.0, 1.0, 1.0), 0.3, 1, pic.PIC_SCHEME_WT, precision=pic.PIC_FP64,
+                  capacity=(n,), tile=(1, 17, 25))
+    orc = oracle.Sim(grid, (1.0, 1.0, 1.0), 0.3, 1, pic.PIC_SCHEME_WT)
+    x = rng.random((3, n)) * np.array(grid)[:, None]
+    run.load(0, 1.0, 1.0, 1.0, x, np.zeros((3, n)))
+    orc.add_species(1.0, 1.0, 1.0, x, np.zeros((3, n)))
+    want = np.max(np.abs(orc.rho()))
+    got = run.diag()
+    assert got["status"] == pic.PIC_OK
+    assert abs(got["max_gauss_residual"] - want) <= 1e-11 * want
+    run.close()
+    orc.close()
